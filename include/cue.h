@@ -96,7 +96,8 @@ typedef struct cue_sim cue_sim;   /* opaque, host-side */
 
 /* ---- options (cue_set_option) ------------------------------------------ */
 #define CUE_OPT_PATH            1  /* value: CUE_PATH_*                                    */
-#define CUE_OPT_TEMPORAL_DEPTH  2  /* value: steps fused per launch on the fused path (1..16),
+#define CUE_OPT_TEMPORAL_DEPTH  2  /* value: steps fused per launch on the fused path, or per
+                                      exchange of the persistent path's tile engine (1..16),
                                       0 = library choice; on 3D handles 2 selects the
                                       blocked path under AUTO, other values the one-step
                                       kernel                                                */
@@ -128,7 +129,10 @@ typedef struct cue_sim cue_sim;   /* opaque, host-side */
 #define CUE_INFO_HELPERS       20  /* helper blocks of the last fused 2D launch: blocks that
                                       share out the cones of crowded tiles (sized from the
                                       crowding the previous run reported; 0 on the first)  */
-#define CUE_PATH_AUTO   0          /* library picks: fused for 2D grids of at least one tile
+#define CUE_PATH_AUTO   0          /* library picks: for 2D grids that fit the SMs' shared
+                                      memory (up to about 1500^2, nx >= 128, any nx), above
+                                      65536 nodes or with nx % 4 != 0, the persistent path's
+                                      tile engine; else fused for 2D grids of at least one tile
                                       per SM; else cluster for 2D grids of at least 4096
                                       nodes with at most 128 cones and 16384 nodes per block;
                                       else resident; else persistent; else plain (3D: one
@@ -141,9 +145,12 @@ typedef struct cue_sim cue_sim;   /* opaque, host-side */
                                       handles (nx % 4 == 0, step_len <= h, at most 512
                                       sources) two steps per launch, a run's odd last step
                                       on the one-step kernel                               */
-#define CUE_PATH_PERSIST 3         /* 2D, nx % 4 == 0: one cooperative launch for the whole
-                                      run; per step one pass over field tiles and cone
-                                      chunks, then a bounded grid barrier                   */
+#define CUE_PATH_PERSIST 3         /* 2D, nx % 4 == 0 (AUTO: any nx): one cooperative launch
+                                      for the whole run.  Grids of nx >= 128 that fit: one tile
+                                      per SM in shared memory, borders exchanged every few
+                                      steps; else (or with CUE_OPT_PERSIST_* set, or inside a
+                                      stream capture) per step one pass over field tiles and
+                                      cone chunks, then a bounded grid barrier              */
 #define CUE_PATH_RESIDENT 4        /* 2D, nx % 4 == 0, both field buffers within one block's
                                       shared memory (128^2: 128 KB), at most 256 cones and
                                       1024 sources: one block holds the grid in shared

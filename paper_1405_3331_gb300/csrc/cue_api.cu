@@ -48,6 +48,17 @@ WorkspaceLayout workspace_layout(const cue_params &p, int n_src, int n_axons)
         w.inter_off = off;
         off += align256(sizeof(float) * (size_t)p.nx * p.ny * p.nz);
     }
+    w.base_total = off;
+    // the tile engine's flags and inboxes, for the 2D grids it can hold
+    if (p.dim == 2 && p.nx >= 128 && (long long)p.nx * p.ny <= kTilesMaxNodes && n_axons <= kTilesMaxCones) {
+        w.tiles_off = off;
+        off += align256(tiles_ctl_bytes());
+        w.tiles_packets_off = off;
+        off += align256(2 * sizeof(unsigned long long) * (size_t)p.nx * p.ny);
+        w.tiles_zero = off - w.tiles_off;
+        w.tiles_inbox_off = off;
+        off += align256(sizeof(int32_t) * 2 * kTilesMax * (size_t)(n_axons > 0 ? n_axons : 0));
+    }
     w.total = off;
     return w;
 }
@@ -129,17 +140,34 @@ int run_coupled(Sim &s, int nsteps)
     s.persist_used = false;
     s.resident_used = false;
     s.cluster_used = false;
-    // AUTO: the temporally blocked kernel when the grid gives every SM a tile;
+    // AUTO, 2D: the persistent path's tile engine ahead of the others for rows that are not whole float4
+    // groups (which otherwise run two scalar launches a step: 1025 x 769 17.4 -> 1.8 us) and for grids above
+    // those the cluster path is kept for (512 x 384 with 2,000 cones 4.3 -> 1.5 us; 1024^2 with a map 6.4 -> 1.6
+    // on the work-list kernel, without one 3.4 -> 1.4 on the fused path), unless the handle's last runs
+    // crowded into few tiles.  Then the temporally blocked kernel when the grid gives every SM a tile;
     // else a cluster of CTAs with the grid in their distributed shared memory
     // where its measured step is the shortest (cluster_preferred); else one
     // block with the grid in shared memory; else the persistent launch (larger
     // small grids, or many cones); else plain.
-    const bool small = !fused_supported(s) || fused_tile_count(s.params) < sm_count_api();
+    const bool fused_ok = fused_supported(s);
+    const bool small = !fused_ok || fused_tile_count(s.params) < sm_count_api();
     int rc = 1;
+    bool tiles = s.path == CUE_PATH_PERSIST;
+    if (s.path == CUE_PATH_AUTO && s.fd.dim == 2 && tiles_supported(s)) {
+        const bool first = !s.vec4 || (long long)s.fd.nx * s.fd.ny > 65536;
+        // (microseconds a step of the path it displaces)
+        const double alt_us = !small ? 4.0 : cluster_preferred(s) ? 2.5 : 6.5;
+        tiles = !s.vec4 || !tiles_crowded(s, alt_us);
+        if (first && tiles) rc = run_tiles_if_supported(s, nsteps);
+        if (rc != 1) return rc;
+        tiles = tiles && small;
+    }
     if (s.path == CUE_PATH_CLUSTER || (s.path == CUE_PATH_AUTO && small && cluster_preferred(s)))
         rc = run_cluster_if_supported(s, nsteps);
     if (rc != 1) return rc;
     if (s.path == CUE_PATH_RESIDENT || (s.path == CUE_PATH_AUTO && small)) rc = run_resident_if_supported(s, nsteps);
+    if (rc != 1) return rc;
+    if (tiles) rc = run_tiles_if_supported(s, nsteps);
     if (rc != 1) return rc;
     if (s.path == CUE_PATH_PERSIST || (s.path == CUE_PATH_AUTO && small)) rc = run_persist_if_supported(s, nsteps);
     if (rc != 1) return rc;
@@ -267,6 +295,19 @@ int cue_init(cue_sim **out, const cue_params *params, const cone_params *cone, f
              const float *d_src_map, float *d_pos, float *d_dir, uint8_t *d_active, int32_t n_axons,
              void *d_workspace, size_t ws_bytes, void *stream)
 {
+    return sim_init(out, params, cone, d_field_a, d_field_b, d_src_cell, d_src_emit, n_src, d_src_map, d_pos, d_dir,
+                    d_active, n_axons, d_workspace, ws_bytes, stream, false);
+}
+
+}  // extern "C"
+
+namespace cue {
+
+int sim_init(cue_sim **out, const cue_params *params, const cone_params *cone, float *d_field_a, float *d_field_b,
+             const int32_t *d_src_cell, const float *d_src_emit, int32_t n_src, const float *d_src_map, float *d_pos,
+             float *d_dir, uint8_t *d_active, int32_t n_axons, void *d_workspace, size_t ws_bytes, void *stream,
+             bool base_only)
+{
     if (!out) return CUE_ERR_ARG;
     *out = nullptr;
     if (!params_ok(params) || !cone_ok(cone)) return CUE_ERR_ARG;
@@ -279,6 +320,10 @@ int cue_init(cue_sim **out, const cue_params *params, const cone_params *cone, f
     ConeDesc cdesc;
     if (make_descs(*params, *cone, fdesc, cdesc) != CUE_OK) return CUE_ERR_UNSTABLE;
     WorkspaceLayout wl = workspace_layout(*params, n_src, n_axons);
+    if (base_only) {
+        wl.total = wl.base_total;
+        wl.tiles_off = 0;
+    }
     if (!d_workspace || ws_bytes < wl.total || (reinterpret_cast<uintptr_t>(d_workspace) & 255u))
         return CUE_ERR_WORKSPACE;
 
@@ -309,6 +354,7 @@ int cue_init(cue_sim **out, const cue_params *params, const cone_params *cone, f
     cudaError_t e = cudaMemsetAsync(s->ws, 0, 256, s->stream);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(s->ws + wl.bin_count_off, 0, wl.bin_list_off - wl.bin_count_off, s->stream);
+    if (e == cudaSuccess && wl.tiles_off) e = cudaMemsetAsync(s->ws + wl.tiles_off, 0, wl.tiles_zero, s->stream);
 
     if (e == cudaSuccess) e = launch_src_xyz(*s);
     if (e != cudaSuccess) {
@@ -318,6 +364,16 @@ int cue_init(cue_sim **out, const cue_params *params, const cone_params *cone, f
     *out = s;
     return CUE_OK;
 }
+
+size_t base_workspace_bytes(const cue_params *params, int32_t n_src, int32_t n_axons)
+{
+    if (!params_ok(params) || n_src < 0 || n_axons < 0) return 0;
+    return workspace_layout(*params, n_src, n_axons).base_total;
+}
+
+}  // namespace cue
+
+extern "C" {
 
 int cue_step(cue_sim *s, int32_t nsteps)
 {
@@ -627,6 +683,11 @@ void cue_destroy(cue_sim *s)
         cudaEventDestroy(s->help_ev);
     }
     if (s->help_host) cudaFreeHost(s->help_host);
+    if (s->crowd_ev) {
+        cudaEventSynchronize(s->crowd_ev);
+        cudaEventDestroy(s->crowd_ev);
+    }
+    if (s->crowd_host) cudaFreeHost(s->crowd_host);
     delete s;
 }
 

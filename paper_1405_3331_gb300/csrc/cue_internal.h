@@ -37,10 +37,29 @@ struct WorkspaceLayout {
     size_t persist_items_cap = 0;
     size_t persist_src_off = 0;  // persistent path: binned sources (PSrc) and their tile keys
     size_t inter_off = 0;        // blocked 3D path: scratch copy of the field's intermediate step (0: none)
+    size_t base_total = 0;       // up to here: everything but the tile engine's part
+    size_t tiles_off = 0;        // tile engine: flags, inbox counts, abort word, post boxes (0: none)
+    size_t tiles_packets_off = 0;  // 2 x cells border packets of 8 bytes
+    size_t tiles_zero = 0;       // bytes from tiles_off that start at zero
+    size_t tiles_inbox_off = 0;  // 2 x kTilesMax x n_axons int32 (cone ids by tile)
     size_t total = 0;
     int n_tiles = 0;
     int bin_cap = 0;             // cone ids per tile bin
 };
+
+// ---- the persistent path's tile engine (k_tiles.cu) ----
+constexpr int kTilesMax = 160;            // tiles (at most one per SM)
+constexpr int kTilesMaxCones = 64 * kTilesMax;   // (its rule's limit) a tile's inbox can hold every cone
+constexpr int kTilesPost = 16;            // cones posted with their state per neighbour and round
+constexpr long long kTilesMaxNodes = 1 << 22;   // grids up to this get its workspace
+struct TilesGeom {
+    int W = 0, R = 0;                     // loaded columns (128 s), rows
+    int HX = 0, HY = 0;                   // halo
+    int gx = 0, gy = 0;                   // tiles per axis
+    int K = 0;                            // steps per round
+    int cap = 0;                          // cones in its shared-memory list
+};
+size_t tiles_ctl_bytes();
 
 // Tile geometry of the fused path.
 struct FusedGeom {
@@ -185,6 +204,17 @@ struct Sim {
     long long persist_limit = 0;  // option: polls before a bounded wait gives up (0 = default)
     int persist_n_items = 0;
     int persist_grid = 0;
+    // its tile engine: the shape for the current depth option, the launches so far (their
+    // parity picks the inbox counts) and a bound on every flag word
+    bool tiles_geom_ready = false, tiles_geom_ok = false;
+    int tiles_geom_depth = 0;
+    TilesGeom tiles_geom{};
+    unsigned tiles_launches = 0, tiles_base = 1;
+    // the most crowded tile of the last watched run (pinned word + event), and the runs left to other paths
+    int *crowd_host = nullptr;
+    cudaEvent_t crowd_ev = nullptr;
+    bool crowd_pending = false;
+    int crowd_skip = 0;
 
     // fused path
     // helper CTAs for crowded tiles: the total need the last run reported, read back
@@ -264,6 +294,19 @@ cudaError_t step_launch(const PInst *d_insts, const PItem *d_chunks, int n_chunk
 int run_persist_if_supported(Sim &s, int nsteps);
 // Coupled steps storing every state (trajectory slot 0 holds the start).
 int run_persist_trajectory(Sim &s, float *traj_field, float *traj_cone, uint32_t step0, int nsteps);
+
+// ---- the persistent path's tile engine (k_tiles.cu) ----
+// Geometry for a grid (depth 0: the library's choice of K); false when no tiling fits.
+bool tiles_geometry(const FieldDesc &f, float step_len, bool map, bool vec, int n_src, int n_axons, int depth, int sms,
+                    TilesGeom &best);
+bool tiles_supported(Sim &s);
+// Whether the handle's last runs were too crowded for it, against another path of alt_us a step.
+bool tiles_crowded(Sim &s, double alt_us);
+// Runs nsteps on the tile engine where it fits: CUE_OK / negative error, or 1 when the caller
+// should use another kernel.
+int run_tiles_if_supported(Sim &s, int nsteps);
+// Coupled steps storing every state, as run_persist_trajectory; 1 when it does not fit.
+int run_tiles_trajectory(Sim &s, float *traj_field, float *traj_cone, uint32_t step0, int nsteps);
 
 // ---- shared-memory resident path for small 2D grids (k_resident.cu) ----
 constexpr int kResThreads = 1024;         // one block: field warps first, then one warp per 32 cones
@@ -385,6 +428,12 @@ cudaError_t blocked_launch(const BInst *d_insts, const int2 *d_items, int n_item
                            int *ids, size_t bin_total, int total_tiles, int *done, unsigned *status,
                            cudaStream_t stream);
 
+// cue_init; base_only: on a workspace of base_workspace_bytes, without the tile engine's part.
+int sim_init(cue_sim **out, const cue_params *params, const cone_params *cone, float *d_field_a, float *d_field_b,
+             const int32_t *d_src_cell, const float *d_src_emit, int32_t n_src, const float *d_src_map, float *d_pos,
+             float *d_dir, uint8_t *d_active, int32_t n_axons, void *d_workspace, size_t ws_bytes, void *stream,
+             bool base_only);
+size_t base_workspace_bytes(const cue_params *params, int32_t n_src, int32_t n_axons);
 // A handle that allocates nothing, not even the pinned word of the helper readback.
 void sim_no_host_alloc(cue_sim *h);
 // ---- coupled steps without the public entry point's checks (cue_api.cu)

@@ -46,15 +46,15 @@ int sim_run_static(const cue_params *params, const cone_params *cone, float *d_f
                    void *stream, int32_t *cur_buffer_out)
 {
     if (!cur_buffer_out || nsteps < 0 || step0 < 0 || step0 + nsteps > 0xFFFFFFFFLL) return CUE_ERR_ARG;
-    const size_t need = cue_workspace_bytes(params, n_src, n_axons);
+    const size_t need = cue::base_workspace_bytes(params, n_src, n_axons);
     if (need == 0) return CUE_ERR_ARG;
     if (need > kStaticScratchBytes) return CUE_ERR_SCRATCH;
     void *ws = nullptr;
     int rc = scratch_for_current_device(&ws);
     if (rc != CUE_OK) return rc;
     cue_sim *h = nullptr;
-    rc = cue_init(&h, params, cone, d_field_a, d_field_b, d_src_cell, d_src_emit, n_src, d_src_map, d_pos, d_dir,
-                  d_active, n_axons, ws, kStaticScratchBytes, stream);
+    rc = cue::sim_init(&h, params, cone, d_field_a, d_field_b, d_src_cell, d_src_emit, n_src, d_src_map, d_pos, d_dir,
+                       d_active, n_axons, ws, kStaticScratchBytes, stream, true);
     if (rc != CUE_OK) return rc;
     cue::sim_no_host_alloc(h);          // no pinned readback word: this entry point allocates nothing
     rc = cue_set_state(h, step0, step0, 0);

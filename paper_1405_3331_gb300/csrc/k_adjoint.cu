@@ -1115,9 +1115,11 @@ int run_adjoint(Sim &s, const float *targets, int nsteps, int k, void *ws, size_
     // its start): one persistent launch where the path runs, else a cone and a
     // field launch per step
     auto trajectory = [&](int len, int64_t nstart) -> int {
-        int rc = (s.path != CUE_PATH_PLAIN && persist_supported(s))
-                     ? run_persist_trajectory(s, sgC, sgP, (uint32_t)nstart, len)
+        int rc = (s.path == CUE_PATH_AUTO || s.path == CUE_PATH_PERSIST)
+                     ? run_tiles_trajectory(s, sgC, sgP, (uint32_t)nstart, len)
                      : 1;
+        if (rc == 1 && s.path != CUE_PATH_PLAIN && persist_supported(s))
+            rc = run_persist_trajectory(s, sgC, sgP, (uint32_t)nstart, len);
         if (rc < 0) return rc;
         for (int m = 0; rc == 1 && m < len; ++m) {
             float *Pm = sgP + 2 * cone_n * m, *Pn = sgP + 2 * cone_n * (m + 1);

@@ -1,0 +1,150 @@
+"""The persistent path's tile engine (csrc/k_tiles.cu) against the plain path, bit for bit:
+both field buffers, the cone state and the cone-update count.  The cases are the edges of its
+range: one and several tiles per axis, rows that are not a multiple of 4 nodes, shifted last
+tiles, one to sixteen steps per round, rounds cut short by the end of a run, a tile with more
+cones than its shared-memory list, cones that all cross tile borders, walls, stops, rate maps
+and the SNR rule."""
+import math
+
+import numpy as np
+import pytest
+
+from paper_1405_3331_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+SNR = dict(gain=8.0, width=2.0, kd=1.5, c_min=0.05, c_max=50.0, turn=math.pi / 30)
+
+
+@pytest.fixture(scope="module")
+def cue():
+    from paper_1405_3331_gb300 import build
+    build.build()
+    from paper_1405_3331_gb300 import cue as binding
+    return binding
+
+
+def _case(name):
+    nx, ny = (int(v) for v in name.split("-")[0].split("x"))
+    tags = name.split("-")[1:]
+    n = next((int(t[:-5]) for t in tags if t.endswith("cones")), 500)
+    w = W.make(name, 2, nx, ny, n_src=0 if "nosrc" in tags else 9, emit=(0.5, 2.0), n_axons=n, C0="smooth", seed=nx + ny,
+               stop_radius=3.0 if "stop" in tags else 0.0, wall_mode=1 if "clamp" in tags else 0,
+               src_map="random" if "map" in tags else False)
+    if "crowd" in tags:                                  # all cones start in a square of 20 nodes
+        rng = np.random.default_rng(nx)
+        w.pos = (np.array([[nx * 0.4], [ny * 0.6]]) + rng.uniform(-10, 10, (2, n))).astype(np.float32)
+    if "inactive" in tags:
+        w.active[::3] = 0
+    return w
+
+
+def _run(cue, w, path, chunks, depth=0, snr=None):
+    sim = cue.Simulation(w, path=path)
+    if depth:
+        sim.set_option(cue.CUE_OPT_TEMPORAL_DEPTH, depth)
+    if snr:
+        sim.set_steering(snr)
+    for k in chunks:
+        sim.sim_run(k)
+    sim.check()
+    out = [f.cpu().numpy() for f in (sim.fields[sim.state()[2]], sim.fields[sim.state()[2] ^ 1])]
+    out += list(sim.snapshot()[1:]) + [sim.state()[2], sim.cone_updates()]
+    info = sim.last_path(), sim.get_option(cue.CUE_INFO_GRID)
+    sim.close()
+    return out, info
+
+
+def _assert_same(a, b):
+    for k, (x, y) in enumerate(zip(a, b)):
+        assert np.array_equal(x, y), f"output {k} differs"
+
+
+@pytest.mark.parametrize("name,chunks", [
+    ("512x300", [1]), ("512x300", [2, 0, 1, 40]), ("257x300-stop", [37]), ("258x300-clamp-map", [37]),
+    ("1025x769-stop-4096cones", [45]), ("640x512-map-clamp-3000cones", [33]), ("1003x131-nosrc", [31]),
+    ("520x400-crowd-clamp-5000cones", [50]), ("517x403-crowd-stop-2500cones", [50]),
+    ("640x400-inactive-clamp", [21]), ("700x500-0cones", [26]),
+])
+def test_tile_engine_equals_plain_bitwise(cue, name, chunks):
+    w = _case(name)
+    a, _ = _run(cue, w, cue.CUE_PATH_PLAIN, chunks)
+    b, (path, grid) = _run(cue, w, cue.CUE_PATH_AUTO, chunks)
+    assert path == cue.CUE_PATH_PERSIST and grid > 1
+    _assert_same(a, b)
+
+
+def test_crowded_runs_go_to_another_path_and_come_back(cue):
+    """4,000 cones in one tile: the run after the first is left to another path (the crowd read
+    back from the first), later ones return; every run gives the plain path's values."""
+    import torch
+    w = _case("1024x640-crowd-clamp-4000cones")
+    a, b = cue.Simulation(w, path=cue.CUE_PATH_PLAIN), cue.Simulation(w)
+    paths = []
+    for k in range(18):
+        for s in (a, b):
+            s.load(C=w.field0(), pos=w.pos, dir=w.dir, active=w.active, step=0)
+            s.sim_run(5 + k % 3)
+            s.check()
+        paths.append(b.last_path())
+        torch.cuda.synchronize()
+        _assert_same(a.snapshot(), b.snapshot())
+    assert paths[0] == cue.CUE_PATH_PERSIST and paths[1] == cue.CUE_PATH_FUSED
+    assert cue.CUE_PATH_PERSIST in paths[2:]
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("depth", [1, 2, 3, 5, 8, 16])
+@pytest.mark.parametrize("name", ["512x384-clamp-2000cones", "263x301-map-stop"])
+def test_any_number_of_steps_per_round(cue, name, depth):
+    w = _case(name)
+    a, _ = _run(cue, w, cue.CUE_PATH_PLAIN, [35])
+    b, (path, _) = _run(cue, w, cue.CUE_PATH_AUTO, [35], depth=depth)
+    assert path == cue.CUE_PATH_PERSIST
+    _assert_same(a, b)
+
+
+@pytest.mark.parametrize("name", ["512x384-clamp-2000cones", "301x263-stop"])
+def test_snr_rule_on_tiles(cue, name):
+    w = _case(name)
+    a, _ = _run(cue, w, cue.CUE_PATH_PLAIN, [30], snr=SNR)
+    b, (path, _) = _run(cue, w, cue.CUE_PATH_AUTO, [30], snr=SNR)
+    assert path == cue.CUE_PATH_PERSIST
+    _assert_same(a, b)
+
+
+@pytest.mark.parametrize("nx,ny", [(512, 300), (261, 300)])
+def test_adjoint_states_on_tiles_are_the_plain_path_s(cue, nx, ny):
+    """The recomputed segments (trajectory mode) against the plain path's, state by state."""
+    w = W.config_c5(seed=3, n=64, n_src=6, n_axons=300, nsteps=40)
+    full = W.make("tr", 2, nx, ny, n_src=6, n_axons=300, wall_mode=1, seed=5, C0="ramp", src_map="zeros", targets=True)
+    assert w.wall_mode == full.wall_mode
+    got = []
+    for path in (cue.CUE_PATH_PLAIN, cue.CUE_PATH_AUTO):
+        sim = cue.Simulation(full, path=path)
+        got.append(sim.adjoint(full.targets, 40, 12, trace=True))
+        sim.check()
+        sim.close()
+    for k in ("trace_C", "trace_cone", "loss"):
+        assert np.array_equal(got[0][k].cpu().numpy(), got[1][k].cpu().numpy()), k
+
+
+def test_device_side_problems_are_reported(cue):
+    """Non-finite input is reported; sources outside the grid are skipped and reported."""
+    w = _case("512x300")
+    w.C0 = w.field0()
+    w.C0[100, 300] = np.nan
+    sim = cue.Simulation(w)
+    sim.sim_run(3)
+    assert sim.last_path() == cue.CUE_PATH_PERSIST
+    assert sim.status() == cue.CUE_ERR_NONFINITE
+    sim.close()
+    w = _case("512x300")
+    w.src_cell = np.array([5, 512 * 300 + 7, -3], np.int32)
+    w.src_emit = np.ones(3, np.float32)
+    sim = cue.Simulation(w)
+    sim.status()
+    sim.sim_run(3)
+    assert sim.status() == cue.CUE_ERR_BOUNDS
+    sim.close()
