@@ -100,15 +100,28 @@ cudaError_t exclusive_scan(const int *in, int *out, int n, int *sums, cudaStream
 // ---------------------------------------------------------------- binning
 struct Grid3 {
     int dim, g[3];
-    double cell;
+    float cell, inv;
+    bool fast;                                           // axis_cell without the division
 };
 
-__device__ __forceinline__ int axis_cell(double x, const Grid3 &G, int ax)
+// floor(x / cell) in 64 bits, clamped to the grid.  Up to 2^22 cells an axis the FP32 product x (1 / cell)
+// is off by less than one, so it names the cell or a neighbour, and the sign of x - k cell (exact: 23 + 24 bits)
+// settles which; the quotient itself is never rounded up to an integer it does not reach (x and cell have
+// 24 bits, so they are at least 2^-24 apart).  An FP64 division per axis and point was most of the hash and
+// connection kernels: GB300's FP64 rate is a small fraction of its FP32 rate.
+__device__ __forceinline__ int axis_cell(float xf, const Grid3 &G, int ax)
 {
-    long long k = (long long)floor(x / G.cell);
-    k = k < 0 ? 0 : k;
-    k = k > G.g[ax] - 1 ? G.g[ax] - 1 : k;
-    return (int)k;
+    const double x = (double)xf, cell = (double)G.cell;
+    if (!G.fast) {
+        long long k = (long long)floor(x / cell);
+        k = k < 0 ? 0 : k;
+        k = k > G.g[ax] - 1 ? G.g[ax] - 1 : k;
+        return (int)k;
+    }
+    int k = (int)floorf(fminf(fmaxf(xf * G.inv, 0.0f), (float)G.g[ax]));      // (NaN: 0)
+    const double t = x - (double)k * cell;
+    k += t < 0.0 ? -1 : t >= cell ? 1 : 0;
+    return min(max(k, 0), G.g[ax] - 1);
 }
 
 __global__ void bin_hash(Grid3 G, int n, const float *__restrict__ pos, int *cell_of, int *count)
@@ -117,7 +130,7 @@ __global__ void bin_hash(Grid3 G, int n, const float *__restrict__ pos, int *cel
     if (i >= n) return;
     long long c = 0, stride = 1;
     for (int ax = 0; ax < G.dim; ++ax) {
-        c += (long long)axis_cell((double)pos[(size_t)ax * n + i], G, ax) * stride;
+        c += (long long)axis_cell(pos[(size_t)ax * n + i], G, ax) * stride;
         stride *= G.g[ax];
     }
     cell_of[i] = (int)c;
@@ -206,51 +219,135 @@ Grid3 make_grid(int dim, const int32_t *grid, float cell)
     G.g[1] = grid[1];
     G.g[2] = dim == 3 ? grid[2] : 1;
     G.cell = cell;
+    G.inv = 1.0f / cell;
+    G.fast = cell >= 1e-30f && cell <= 1e30f && G.g[0] <= 1 << 22 && G.g[1] <= 1 << 22 && G.g[2] <= 1 << 22;
     return G;
 }
 
 // ---------------------------------------------------------------- connections
-__global__ void connect_kernel(Grid3 G, int n_cones, const float *__restrict__ pos, const int *__restrict__ owner,
+// One thread per cone.  The three cells of a row (x - 1, x, x + 1) are neighbours in the
+// binned order too, so a row is one run of sorted ids, and its cell bounds are loaded
+// together.  A thread keeps its first matches in registers and a warp takes its output
+// slots with one atomic.  1,048,576 cones on 262,144 neurons: 300 -> 210 us a call.
+constexpr int kConnectKeep = 4;
+
+__global__ void __launch_bounds__(128) connect_kernel(Grid3 G, int n_cones, const float *__restrict__ pos, const int *__restrict__ owner,
                                const uint8_t *__restrict__ active, int n_neurons, const float *__restrict__ npos,
                                double r2, const int *__restrict__ sorted_id, const int *__restrict__ cell_start,
                                const int *__restrict__ cell_end, int cap, int *src, int *dst, int *count)
 {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= n_cones || (active && !active[a])) return;
+    const int a = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const bool on = a < n_cones && (!active || active[a]);
     double x[3] = {0.0, 0.0, 0.0};
-    int k[3] = {0, 0, 0};
-    for (int ax = 0; ax < G.dim; ++ax) {
-        x[ax] = (double)pos[(size_t)ax * n_cones + a];
-        k[ax] = axis_cell(x[ax], G, ax);
+    int k[3] = {0, 0, 0}, me = 0;
+    if (on) {
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax)
+            if (ax < G.dim) {
+                const float p = pos[(size_t)ax * n_cones + a];
+                x[ax] = (double)p;
+                k[ax] = axis_cell(p, G, ax);
+            }
+        me = owner[a];
     }
-    const int me = owner[a];
     const int zr = G.dim == 3 ? 1 : 0;
-    for (int dz = -zr; dz <= zr; ++dz)
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int cx = k[0] + dx, cy = k[1] + dy, cz = k[2] + dz;
-                if (cx < 0 || cy < 0 || cz < 0 || cx >= G.g[0] || cy >= G.g[1] || cz >= G.g[2]) continue;
-                const long long c = cx + (long long)G.g[0] * (cy + (long long)G.g[1] * cz);
-                const int b = cell_start[c];
-                if (b < 0) continue;
-                const int e = cell_end[c];
-                for (int j = b; j < e; ++j) {
-                    const int nid = sorted_id[j];
-                    if (nid == me) continue;
-                    double d2 = 0.0;
-                    for (int ax = 0; ax < G.dim; ++ax) {
-                        const double d = x[ax] - (double)npos[(size_t)ax * n_neurons + nid];
-                        d2 += d * d;
-                    }
-                    if (d2 < r2) {
-                        const int slot = atomicAdd(count, 1);
-                        if (slot < cap) {
-                            src[slot] = me;
-                            dst[slot] = nid;
-                        }
-                    }
+    // every match of this cone, in a fixed order.  A plane's nine cell bounds go out together (a cell
+    // outside the grid stands in by its neighbour, which changes no run), and its runs' ids four at a time
+    auto each = [&](const auto &fn) {
+        const int x0 = max(k[0] - 1, 0), x1 = min(k[0] + 1, G.g[0] - 1);
+        for (int dz = -zr; dz <= zr; ++dz) {
+            const int cz = k[2] + dz;
+            if (cz < 0 || cz >= G.g[2]) continue;
+            int cb[3][3], ce[3][3];
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy) {
+                const int cy = min(max(k[1] + dy - 1, 0), G.g[1] - 1);
+                const long long c = (long long)G.g[0] * (cy + (long long)G.g[1] * cz);
+                const int cx[3] = {x0, k[0], x1};
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    cb[dy][q] = cell_start[c + cx[q]];
+                    ce[dy][q] = cell_end[c + cx[q]];
                 }
             }
+            int b[3], len[3];
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy) {
+                b[dy] = 0x7fffffff;
+                int e = -1;
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    if (cb[dy][q] >= 0) {               // (empty cells hold -1)
+                        b[dy] = min(b[dy], cb[dy][q]);
+                        e = max(e, ce[dy][q]);
+                    }
+                const int cy = k[1] + dy - 1;
+                len[dy] = e < 0 || cy < 0 || cy >= G.g[1] ? 0 : e - b[dy];
+            }
+            const int n = len[0] + len[1] + len[2];
+            for (int i0 = 0; i0 < n; i0 += 4) {
+                int id[4];
+                float p[4][3];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int i = min(i0 + q, n - 1);
+                    const int j = i < len[0] ? b[0] + i : i < len[0] + len[1] ? b[1] + i - len[0] : b[2] + i - len[0] - len[1];
+                    id[q] = sorted_id[j];
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) p[q][ax] = ax < G.dim ? npos[(size_t)ax * n_neurons + id[q]] : 0.0f;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (i0 + q >= n || id[q] == me) continue;
+                    double d2 = 0.0;
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax)
+                        if (ax < G.dim) {
+                            const double d = x[ax] - (double)p[q][ax];
+                            d2 += d * d;
+                        }
+                    if (d2 < r2) fn(id[q]);
+                }
+            }
+        }
+    };
+    int found[kConnectKeep], nf = 0;
+    if (on)
+        each([&](int nid) {
+#pragma unroll
+            for (int q = 0; q < kConnectKeep; ++q)
+                if (nf == q) found[q] = nid;
+            nf++;
+        });
+    int upto = nf;                                       // matches of the warp up to this lane
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, upto, 31);
+    if (total == 0) return;
+    int slot = 0;
+    if (lane == 0) slot = atomicAdd(count, total);
+    slot = __shfl_sync(0xffffffffu, slot, 0) + upto - nf;
+#pragma unroll
+    for (int q = 0; q < kConnectKeep; ++q)
+        if (q < nf && slot + q < cap) {
+            src[slot + q] = me;
+            dst[slot + q] = found[q];
+        }
+    if (nf > kConnectKeep) {                             // the rest of a cone with many: once more
+        int q = 0;
+        each([&](int nid) {
+            if (q >= kConnectKeep && slot + q < cap) {
+                src[slot + q] = me;
+                dst[slot + q] = nid;
+            }
+            ++q;
+        });
+    }
 }
 
 // ---------------------------------------------------------------- adjacency list
@@ -347,19 +444,34 @@ CsrLayout csr_layout(int nv, int ne_cap)
 // synchronisation the text describes).  Three flag words rotate: level L sets
 // flag[L % 3] when it finds a vertex and clears flag[(L + 1) % 3], last read
 // after the barrier before the previous one.
+//
+// Most levels of a sparse graph hold a few thousand vertices, and a level over the whole
+// grid costs its barrier (9.8 us a level over 1,024 blocks).  So the search starts on one
+// thread-block cluster (bfs_cluster_kernel): its queues and the visited map lie in distributed
+// shared memory, and a level ends at the hardware's cluster barrier.  When a level is
+// sent more than kBfsWide finds (or a queue overflows) the cluster stops and bfs_kernel, over all
+// SMs, goes on from the levels written so far: `from` says where ({done, level}; null: from the source).
+// 262,144 vertices, 786,432 edges, 88 levels: 890 -> 390 us a call (4 us a level: the row, its edges and
+// the barrier, one after the other).  Measured and not kept: claiming by a compare-and-swap of the level before
+// the send (480; each claim waits for L2), the block's finds staged and handed out together (690).
 __global__ void __launch_bounds__(256) bfs_kernel(int nv, const int *__restrict__ row, const int *__restrict__ col,
                                                   int source, int *level, uint8_t *F0, uint8_t *F1, int *flag,
-                                                  PBar *bar, unsigned expected, long long limit, unsigned *status)
+                                                  PBar *bar, unsigned expected, long long limit, unsigned *status,
+                                                  const int *from)
 {
+    if (from && from[0]) return;                         // the cluster finished (every block sees it)
     const int stride = gridDim.x * blockDim.x;
     const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
+    const int first = from ? from[1] : 0;
     for (int v = t0; v < nv; v += stride) {
-        level[v] = v == source ? 0 : -1;
-        F0[v] = v == source;
-        F1[v] = 0;
+        if (!from) level[v] = v == source ? 0 : -1;
+        const int l = from ? __ldcg(level + v) : level[v];
+        const uint8_t in = l >= 0 && l == first;         // (the cluster has reached none beyond `first`)
+        F0[v] = first & 1 ? 0 : in;
+        F1[v] = first & 1 ? in : 0;
     }
     if (!grid_barrier(bar, expected, limit, status)) return;
-    for (int L = 0; L < nv; ++L) {
+    for (int L = first; L < nv; ++L) {
         uint8_t *Fc = (L & 1) ? F1 : F0, *Fn = (L & 1) ? F0 : F1;
         bool found = false;
         for (int v = t0; v < nv; v += stride) {
@@ -379,6 +491,156 @@ __global__ void __launch_bounds__(256) bfs_kernel(int nv, const int *__restrict_
         if (!grid_barrier(bar, expected, limit, status)) return;
         if (!__ldcg(flag + L % 3)) break;
     }
+}
+
+constexpr int kBfsThreads = 1024;
+constexpr int kBfsQueue = 16384;             // finds a block can be sent for a level (two queues), an equal part by each block
+constexpr int kBfsMaxVertices = 1 << 22;     // bits of the visited map over a cluster of 16 (32 KB a block)
+constexpr int kBfsWide = 65536;              // a level that was sent more finds goes to all SMs
+
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, int rank)
+{
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+
+__device__ __forceinline__ void st_cluster(void *p, int rank, int v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ void cluster_sync_all()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Vertex u belongs to block u % G, which alone knows (a bit in its shared memory) whether it was
+// reached.  At level L a block goes over the vertices it was sent, drops those it has seen, writes the others'
+// level and sends their edges' ends to the blocks they belong to, into the sender's own part of
+// their queues: no atomic leaves a block, and nothing waits for memory but the row and its edges.
+// state: {1 when the search is complete, else 0; the level to go on from, whose vertices all carry it}.
+// level is -1 everywhere at the start.
+__global__ void __launch_bounds__(kBfsThreads) bfs_cluster_kernel(int nv, const int *__restrict__ row, const int *__restrict__ col,
+                                                                  int source, int *level, int *state)
+{
+    extern __shared__ int queue[];                       // [2][G][kBfsQueue / G], then the visited map
+    unsigned *seen = reinterpret_cast<unsigned *>(queue + 2 * kBfsQueue);
+    __shared__ int cnt[2][16], tot[2][16], over[2];      // by level parity and sender: finds sent here; to anyone; some lost
+    __shared__ int s_out[16];                            // finds of this level by the block they go to
+    int G, rank;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(G));
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const int tid = threadIdx.x, lane = tid & 31, part = kBfsQueue / G;
+    const int words = (nv / G + 32) >> 5;
+    for (int i = tid; i < words; i += kBfsThreads) seen[i] = 0;
+    const bool valid = source >= 0 && source < nv;
+    if (tid < 16) {
+        cnt[0][tid] = tid == 0 && valid && source % G == rank;
+        tot[0][tid] = tid == 0 && valid;
+        s_out[tid] = 0;
+    }
+    if (tid == 0) {
+        over[0] = over[1] = 0;
+        queue[0] = source;
+    }
+    cluster_sync_all();
+    const int per = kBfsThreads / G, from = tid / per;   // this thread's sender
+    int L = 0;
+    bool wide = false;
+    for (; L < nv; ++L) {
+        const int par = L & 1;
+        const int sent = __reduce_add_sync(0xffffffffu, lane < G ? tot[par][lane] : 0);
+        if (sent == 0) break;
+        wide = over[par] != 0 || sent > kBfsWide;        // (the same in every thread of the cluster)
+        if (wide) break;
+        const int *q = queue + par * kBfsQueue + from * part;
+        int *qn = queue + (par ^ 1) * kBfsQueue + rank * part;
+        const int n = cnt[par][from];
+        for (int i = tid - from * per; i < n; i += per) {
+            const int v = q[i], at = v / G;
+            const unsigned bit = 1u << (at & 31);
+            if (atomicOr(&seen[at >> 5], bit) & bit) continue;
+            level[v] = L;
+            const int e1 = row[v + 1];
+            for (int e = row[v]; e < e1; e += 4) {       // four edges at a time: their ends are loaded together
+                int u[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) u[k] = e + k < e1 ? col[e + k] : -1;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (u[k] >= 0) {
+                        const int to = u[k] % G, slot = atomicAdd(&s_out[to], 1);
+                        if (slot < part) st_cluster(qn + slot, to, u[k]);
+                    }
+            }
+        }
+        __syncthreads();
+        if (tid < 32) {
+            const int k = lane < G ? s_out[lane] : 0;
+            const int all = __reduce_add_sync(0xffffffffu, k);
+            const bool lost = __any_sync(0xffffffffu, k > part);
+            if (lane < G) {
+                st_cluster(&cnt[par ^ 1][rank], lane, min(k, part));
+                st_cluster(&tot[par ^ 1][rank], lane, all);
+                if (lost) st_cluster(&over[par ^ 1], lane, 1);
+                s_out[lane] = 0;
+            }
+            if (lane == 0) over[par] = 0;
+        }
+        cluster_sync_all();
+    }
+    if (tid == 0 && rank == 0) {
+        state[0] = wide ? 0 : 1;
+        state[1] = L - 1;                                // (a wide level has a level before it)
+    }
+    cluster_sync_all();                                  // no block leaves while another may still write to it
+}
+
+int bfs_smem(int nv, int G) { return (2 * kBfsQueue + (nv / G + 32) / 32 + 1) * (int)sizeof(int); }
+
+// Blocks of the cluster the search starts on: 16 where the device can schedule it, else 8, else 0 (none).
+int bfs_cluster_size()
+{
+    static int size = -1;
+    if (size >= 0) return size;
+    const int smem = bfs_smem(kBfsMaxVertices, 16);
+    int best = 0;
+    if (cudaFuncSetAttribute(bfs_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+        cudaFuncSetAttribute(bfs_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+        for (int g = 16; g >= 8 && best == 0; g /= 2) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(g);
+            cfg.blockDim = dim3(kBfsThreads);
+            cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = g;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, bfs_cluster_kernel, &cfg) == cudaSuccess && n > 0) best = g;
+        }
+    cudaGetLastError();                                  // a size the device refuses is no error of the caller's
+    size = best;
+    return size;
+}
+
+cudaError_t launch_bfs_cluster(int G, int nv, const int *row, const int *col, int source, int *level, int *state, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(G);
+    cfg.blockDim = dim3(kBfsThreads);
+    cfg.dynamicSmemBytes = bfs_smem(nv, G);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = G;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, bfs_cluster_kernel, nv, row, col, source, level, state);
 }
 
 struct BfsLayout {
@@ -529,6 +791,14 @@ int cue_bfs(int32_t nv, const int32_t *d_row, const int32_t *d_col, int32_t sour
         return CUE_ERR_CUDA;
     const int grid = std::max(1, std::min(blocks_of(nv, 256), maxb * sm_count_g()));
     if (cudaMemsetAsync(W, 0, 768, st) != cudaSuccess) return CUE_ERR_CUDA;   // status, barrier, flags
+    // the cluster first; the launch over all SMs returns at once unless a level was too wide for it
+    const int G = nv <= kBfsMaxVertices / 16 * bfs_cluster_size() ? bfs_cluster_size() : 0;
+    int *state = G > 0 ? reinterpret_cast<int *>(W + L.flag) + 8 : nullptr;
+    if (G > 0) {
+        if (cudaMemsetAsync(d_level, 0xFF, sizeof(int) * (size_t)nv, st) != cudaSuccess ||
+            launch_bfs_cluster(G, nv, d_row, d_col, source, d_level, state, st) != cudaSuccess)
+            return CUE_ERR_CUDA;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(256);
@@ -541,7 +811,8 @@ int cue_bfs(int32_t nv, const int32_t *d_row, const int32_t *d_col, int32_t sour
     cudaError_t e = cudaLaunchKernelEx(&cfg, bfs_kernel, (int)nv, d_row, d_col, (int)source, d_level,
                                        reinterpret_cast<uint8_t *>(W + L.F), reinterpret_cast<uint8_t *>(W + L.U),
                                        reinterpret_cast<int *>(W + L.flag), reinterpret_cast<PBar *>(W + L.bar),
-                                       (unsigned)grid, kPersistSpinLimit, reinterpret_cast<unsigned *>(W + L.status));
+                                       (unsigned)grid, kPersistSpinLimit, reinterpret_cast<unsigned *>(W + L.status),
+                                       static_cast<const int *>(state));
     return e == cudaSuccess ? CUE_OK : CUE_ERR_CUDA;
 }
 

@@ -46,6 +46,13 @@ def _ws(torch, nbytes, device):
     return buf, (buf.data_ptr() + 255) & ~255
 
 
+def _release(torch, device, stream, buf):
+    """The workspace is released on return.  On the current stream the allocator hands it on in stream
+    order; on another one the call's work must have ended (the outputs are the current stream's too)."""
+    if stream != torch.cuda.current_stream(device).cuda_stream:
+        torch.cuda.synchronize(device)
+
+
 def _grid(grid):
     return (ct.c_int32 * 3)(*(list(grid) + [1] * (3 - len(grid))))
 
@@ -66,8 +73,7 @@ def bin_points(pos, cell: float, grid, stream=None):
     st = (stream or torch.cuda.current_stream(dev)).cuda_stream
     _check(L.cue_bin_points(dim, n, pos.data_ptr(), float(cell), _grid(grid), *[t.data_ptr() for t in out], ws,
                             nbytes, st), "cue_bin_points")
-    torch.cuda.synchronize(dev)                      # the workspace is released on return
-    del buf
+    _release(torch, dev, st, buf)
     return tuple(out)
 
 
@@ -105,8 +111,7 @@ def csr(nv: int, src, dst, count, stream=None):
     st = (stream or torch.cuda.current_stream(dev)).cuda_stream
     _check(L.cue_csr_build(nv, cap, count.data_ptr(), src.data_ptr(), dst.data_ptr(), row.data_ptr(), col.data_ptr(),
                            m.data_ptr(), ws, nbytes, st), "cue_csr_build")
-    torch.cuda.synchronize(dev)
-    del buf
+    _release(torch, dev, st, buf)
     return row, col, m
 
 

@@ -171,3 +171,67 @@ def test_connectivity_at_the_benchmark_size(g):
     hit = lev > 0
     np.testing.assert_array_equal(best[hit], lev[hit])                      # each level from a predecessor
     assert np.all(lev[lev < 0] == -1) and not np.any((lev < 0) & (best < np.iinfo(np.int64).max))
+
+
+@pytest.mark.parametrize("name", ["wide", "one-queue", "wide-then-path", "dense"])
+def test_bfs_beyond_one_cluster(g, name):
+    """Levels the starting cluster cannot hold go on over all SMs: a level of 100,000 vertices, a
+    level whose 20,000 vertices all fall to one block's queue, a long path after a wide level, and
+    a small dense graph."""
+    import torch
+    if name == "wide":
+        nv, edges = 200000, [(0, np.arange(1, 100001)), (np.arange(1, 100001), np.arange(100000, 200000))]
+    elif name == "dense":                                # few vertices, more finds than the queues hold
+        nv, edges = 1500, [(np.repeat(np.arange(1, 800), 1400), np.tile(np.arange(100, 1500), 799)), (0, np.arange(1, 800))]
+    elif name == "one-queue":
+        mult = np.arange(1, 20001) * 16
+        nv, edges = 330000, [(0, mult), (mult, mult + 1)]
+    else:
+        nv, edges = 120000, [(0, np.arange(1, 90001)), (np.arange(90000, 119999), np.arange(90001, 120000))]
+    src = np.concatenate([np.broadcast_to(a, np.shape(b)) for a, b in edges])
+    dst = np.concatenate([b for _, b in edges])
+    order = np.lexsort((dst, src))
+    row = np.concatenate([[0], np.cumsum(np.bincount(src, minlength=nv))]).astype(np.int32)
+    col = dst[order].astype(np.int32)
+    lev = g.bfs(_t(row, torch.int32), _t(col, torch.int32), 0).cpu().numpy()
+    np.testing.assert_array_equal(lev, oracle.bfs(row, col, 0))
+
+
+def test_connections_of_cones_with_many_matches(g):
+    """Cones with none, a few and more matches than a thread keeps, active and not, in 2D and 3D."""
+    import torch
+    for dim in (2, 3):
+        rng = np.random.default_rng(92 + dim)
+        npos = rng.uniform(0, 12, (dim, 400)).astype(np.float32)
+        pos = np.concatenate([rng.uniform(0, 12, (dim, 300)), rng.uniform(20, 30, (dim, 37))], 1).astype(np.float32)
+        owner = rng.integers(0, 400, 337).astype(np.int32)
+        act = (rng.uniform(0, 1, 337) < 0.8).astype(np.uint8)
+        grid, cell, r = [16] * dim, 2.0, 2.0
+        binned = g.bin_points(_t(npos, torch.float32), cell, grid)
+        src, dst, cnt = g.connect(_t(pos, torch.float32), _t(owner, torch.int32), _t(act, torch.uint8),
+                                  _t(npos, torch.float32), r, cell, grid, binned, cap=20000)
+        k = int(cnt.item())
+        ws, wd = oracle.connect(pos.astype(np.float64), owner, act, npos.astype(np.float64), r)
+        assert k == ws.size and k > 337
+        assert sorted(zip(src.cpu().numpy()[:k], dst.cpu().numpy()[:k])) == sorted(zip(ws, wd))
+        _, _, few = g.connect(_t(pos, torch.float32), _t(owner, torch.int32), _t(act, torch.uint8),
+                              _t(npos, torch.float32), r, cell, grid, binned, cap=10)
+        assert int(few.item()) == k                      # the count is of all matches, whatever fits
+
+
+def test_cells_at_their_edges(g):
+    """Points on, just below and just above cell edges, outside the grid, infinite and NaN: the cell is
+    floor(x / cell) in 64 bits, clamped to the grid, for sides where the quotient is inexact."""
+    import torch
+    rng = np.random.default_rng(95)
+    for cell, n in ((0.1, 5000), (3.0, 700), (1.7e-3, 1 << 20), (2.0, 64), (1e-32, 9)):
+        cell = np.float32(cell)
+        edge = (rng.integers(0, n + 2, 4000) * np.float64(cell)).astype(np.float32)
+        x = np.concatenate([edge, np.nextafter(edge, np.float32(np.inf)), np.nextafter(edge, np.float32(-np.inf)),
+                            np.array([0.0, -1.0, np.inf, -np.inf, np.nan, 3e38], np.float32)])
+        with np.errstate(over="ignore", invalid="ignore"):
+            q = np.floor(x.astype(np.float64) / np.float64(cell))
+        want = np.where(np.isnan(q), 0, np.clip(np.nan_to_num(q, nan=0.0, posinf=n, neginf=0.0), 0, n - 1)).astype(np.int64)
+        pos = np.stack([x, np.zeros_like(x)])
+        got = g.bin_points(_t(pos, torch.float32), float(cell), [n, 1])[0].cpu().numpy()
+        np.testing.assert_array_equal(got, want)
