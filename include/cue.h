@@ -138,7 +138,8 @@ typedef struct cue_sim cue_sim;   /* opaque, host-side */
                                       else resident; else persistent; else plain (3D: one
                                       launch per step)                                     */
 #define CUE_PATH_PLAIN  1          /* one launch per half-step: cone kernel, field kernel
-                                      (3D with nx % 4 == 0: one launch per step)           */
+                                      (3D with nx % 4 == 0: one launch per step; under AUTO
+                                      grids of any other row length too)                    */
 #define CUE_PATH_FUSED  2          /* temporally blocked field + cones in one kernel (2D:
                                       nx % 4 == 0, no rate map, at most 65536 sources and
                                       256 in any tile's loaded region); on 3D

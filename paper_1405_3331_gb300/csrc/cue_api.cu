@@ -175,7 +175,7 @@ int run_coupled(Sim &s, int nsteps)
     if (rc != 1) return rc;
     rc = run_fused_if_supported(s, nsteps);
     if (rc != 1) return rc;       // handled (0 = ok, < 0 = error)
-    // 3D with the TMA field kernel: cones, field and sources of a step in one launch
+    // 3D with the TMA field kernel, and (AUTO) grids of any row length: cones, field and sources of a step in one launch
     const bool merged3 = s.fd.dim == 3 && s.vec4 && field3d_tma_prepare(s);
     for (int k = 0; k < nsteps; ++k) {
         float *in = s.field[s.cur], *out = s.field[s.cur ^ 1];
@@ -188,6 +188,10 @@ int run_coupled(Sim &s, int nsteps)
             s.launches++;
             // what the launch did not take: the cones read `in`, which no launch of this step writes
             if (e == cudaSuccess && !cones) e = launch_cone_step(s, in, (uint32_t)s.cone_step);
+            if (e == cudaSuccess && !sources) e = launch_sources(s, out);
+        } else if (!s.vec4 && s.path == CUE_PATH_AUTO) {
+            bool sources = false;
+            e = launch_step_any(s, in, out, &sources);
             if (e == cudaSuccess && !sources) e = launch_sources(s, out);
         } else {
             e = launch_cone_step(s, in, (uint32_t)s.cone_step);

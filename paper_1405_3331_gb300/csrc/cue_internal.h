@@ -449,6 +449,9 @@ cudaError_t launch_endpoint_loss(Sim &s, const float *targets, float *loss);
 // One field step Cin -> Cout.  With `sources_done` non-null the kernel may also
 // add the point sources; *sources_done tells whether it did.
 cudaError_t launch_field_step(Sim &s, const float *Cin, float *Cout, bool *sources_done = nullptr);
+// One coupled step on grids of any row length and alignment: cones, field and (where *sources_done says so)
+// sources in one launch.
+cudaError_t launch_step_any(Sim &s, const float *Cin, float *Cout, bool *sources_done);
 // Field step followed by the point sources (in the same kernel where it can).
 cudaError_t launch_field_and_sources(Sim &s, const float *Cin, float *Cout);
 cudaError_t launch_sources(Sim &s, float *Cout);

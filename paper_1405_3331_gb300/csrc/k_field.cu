@@ -8,6 +8,8 @@
 //          [+ dt * M_i] [+ e_k at source nodes]
 // evaluated as beta C_i + alpha sum_j C_j with a missing neighbour (wall)
 // replaced by the node itself (node_update2/3).
+#include <algorithm>
+
 #include "cue_internal.h"
 
 namespace cue {
@@ -206,39 +208,136 @@ __global__ void __launch_bounds__(32 * BY) field3d_vec4(FieldDesc f, const float
 }
 
 // ---------------------------------------------------------------- any size
-// One thread per node; used when nx is not a multiple of 4 or a buffer is not
-// 16-byte aligned.
-template <bool MAP>
-__global__ void __launch_bounds__(256) field_scalar(FieldDesc f, const float *__restrict__ Cin,
-                                                    float *__restrict__ Cout,
-                                                    const float *__restrict__ M, unsigned *status)
+// Any row length and alignment (nx not a multiple of 4, or a buffer that is not 16-byte aligned): one
+// thread per column of the march (y in 2D, z in 3D), so a node's index is worked out once
+// per thread and its neighbours along the march stay in registers; the others come from L1.  A launch
+// can carry the step's cones (blocks at the start of the grid, kAnyCones each: their chain of dependent loads is the
+// longest) and the point sources of its nodes (added once the block's nodes are stored), so a
+// coupled step is one launch, and a programmatic dependent one: its blocks are set up while the previous step's
+// end.  129 x 97 x 65 with 5,000 cones: 17.3 us a step as three launches with two 64-bit divisions per node
+// -> 5.4 (5.3 of it the field's); 255^3 86 -> 69; 2D 2049^2 with 16,384 cones 31 -> 9.3, 4095^2 89 -> 37.
+// What bounds it: rows that start anywhere in a sector, so every warp's load and store touches one
+// more, and the loads of a step behind the stores of the one before.  Measured and not kept: tiles of 32 x 8
+// columns in 3D (6.0), four march steps loaded ahead of their stores (5.6; 4095^2 60).
+constexpr int kAnyCones = 128;
+constexpr int kAnySources = 1024;             // point sources a block looks through
+
+struct AnyArgs {
+    FieldDesc f;
+    ConeDesc c;
+    const float *Cin;
+    float *Cout;
+    const float *M;
+    int chunk;                                // march steps per block
+    unsigned plane_blocks, cone_blocks;
+    // cones
+    uint32_t step;
+    int n;
+    float *pos, *dir;
+    uint8_t *active;
+    const float *src_xyz;
+    int n_stop;
+    unsigned long long *counter;
+    // point sources
+    const int32_t *src_cell;
+    const float *src_emit;
+    int n_add;
+    unsigned *status;
+};
+
+// A weak load that the compiler may move past this kernel's stores (they go to another buffer), but
+// not before the dependency wait: the pointer carries the wait's result.
+__device__ __forceinline__ float ld_in(const float *p)
 {
-    const size_t n = (size_t)f.nx * f.ny * f.nz;
-    const size_t sy = f.nx, sz = (size_t)f.nx * f.ny;
-    bool bad = false;
-    for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
-         c += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(c % f.nx);
-        const int j = (int)((c / f.nx) % f.ny);
-        const int k = (int)(c / sz);
-        const float ci = __ldg(Cin + c);
-        const float xm = i > 0 ? __ldg(Cin + c - 1) : ci;
-        const float xp = i < f.nx - 1 ? __ldg(Cin + c + 1) : ci;
-        const float ym = j > 0 ? __ldg(Cin + c - sy) : ci;
-        const float yp = j < f.ny - 1 ? __ldg(Cin + c + sy) : ci;
-        float o;
-        if (f.dim == 3) {
-            const float zm = k > 0 ? __ldg(Cin + c - sz) : ci;
-            const float zp = k < f.nz - 1 ? __ldg(Cin + c + sz) : ci;
-            o = node_update3(ci, xm, xp, ym, yp, zm, zp, f.alpha, f.beta);
-        } else {
-            o = node_update2(ci, xm, xp, ym, yp, f.alpha, f.beta);
+    float v;
+    asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
+template <int DIM, bool MAP>
+__global__ void __launch_bounds__(256) step_any(const __grid_constant__ AnyArgs A)
+{
+    const FieldDesc &f = A.f;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const size_t plane = DIM == 3 ? (size_t)f.nx * f.ny : (size_t)f.nx;
+    const int tid = threadIdx.x;
+    long long after;                          // 0, once the previous launch's writes are visible
+    if (blockIdx.x < A.cone_blocks) {
+        asm volatile("griddepcontrol.wait;\n mov.u64 %0, 0;" : "=l"(after)::"memory");
+        if (tid >= kAnyCones) return;
+        const float *C = A.Cin + after;
+        const int a = blockIdx.x * kAnyCones + tid, n = A.n;
+        const bool inr = a < n;
+        const uint8_t act = inr ? A.active[a] : 0;
+        float p[DIM], d[DIM], xi[DIM];
+#pragma unroll
+        for (int i = 0; i < DIM; ++i) {
+            p[i] = inr ? A.pos[(size_t)i * n + a] : 0.0f;
+            d[i] = inr ? A.dir[(size_t)i * n + a] : 0.0f;
         }
-        if constexpr (MAP) o = fmaf(f.dt, __ldg(M + c), o);
-        bad |= !(fabsf(o) <= 3.402823466e38f);
-        Cout[c] = o;
+        cone_noise<DIM>(A.c.key0, A.c.key1, (uint32_t)a, A.step, xi);
+        const bool live = inr && act;
+        count_active(A.counter, live);
+        if (!live) return;
+        auto ld = [&](int i, int j, int k) { return ld_in(C + (size_t)i + (size_t)f.nx * j + (DIM == 3 ? plane * k : 0)); };
+        const bool alive = cone_step_rule<DIM>(f, A.c, ld, xi, p, d, A.src_xyz, A.n_stop, A.n_stop);
+        bool bad = false;
+#pragma unroll
+        for (int i = 0; i < DIM; ++i) {
+            A.pos[(size_t)i * n + a] = p[i];
+            A.dir[(size_t)i * n + a] = d[i];
+            bad |= !(fabsf(p[i]) <= 3.402823466e38f) || !(fabsf(d[i]) <= 3.402823466e38f);
+        }
+        if (!alive) A.active[a] = 0;
+        if (bad) flag_status(A.status, kStatusNonFinite);
+        return;
     }
-    if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) flag_status(status, kStatusNonFinite);
+    const unsigned fb = blockIdx.x - A.cone_blocks, pb = fb % A.plane_blocks, cb = fb / A.plane_blocks;
+    const size_t i0 = (size_t)pb * 256, i = i0 + tid;
+    const int N = DIM == 3 ? f.nz : f.ny;
+    const int z0 = (int)cb * A.chunk, z1 = min(z0 + A.chunk, N);
+    const bool in = i < plane;
+    const unsigned y = DIM == 3 ? (unsigned)i / (unsigned)f.nx : 0u, x = (unsigned)i - y * (unsigned)f.nx;
+    const ptrdiff_t xm = x > 0 ? -1 : 0, xp = x + 1 < (unsigned)f.nx ? 1 : 0;
+    const ptrdiff_t ym = DIM == 3 && y > 0 ? -(ptrdiff_t)f.nx : 0, yp = DIM == 3 && y + 1 < (unsigned)f.ny ? (ptrdiff_t)f.nx : 0;
+    asm volatile("griddepcontrol.wait;\n mov.u64 %0, 0;" : "=l"(after)::"memory");
+    bool bad = false;
+    if (in) {
+        const float *C = A.Cin + after + plane * z0 + i;
+        float *O = A.Cout + plane * z0 + i;
+        const float *M = MAP ? A.M + plane * z0 + i : nullptr;
+        float c = ld_in(C), m = z0 > 0 ? ld_in(C - plane) : c;
+#pragma unroll 4
+        for (int z = z0; z < z1; ++z, C += plane, O += plane) {
+            const float p = z + 1 < N ? ld_in(C + plane) : c;
+            const float l = ld_in(C + xm), r = ld_in(C + xp);
+            float o;
+            if constexpr (DIM == 3) o = node_update3(c, l, r, ld_in(C + ym), ld_in(C + yp), m, p, f.alpha, f.beta);
+            else o = node_update2(c, l, r, m, p, f.alpha, f.beta);
+            if constexpr (MAP) {
+                o = fmaf(f.dt, __ldg(M), o);
+                M += plane;
+            }
+            bad |= !(fabsf(o) <= 3.402823466e38f);
+            *O = o;
+            m = c;
+            c = p;
+        }
+    }
+    if (__any_sync(0xffffffffu, bad) && (tid & 31) == 0) flag_status(A.status, kStatusNonFinite);
+    if (A.n_add > 0) {
+        __syncthreads();                      // the block's nodes are stored: their sources (atomic: duplicates add up)
+        const long long n_cells = (long long)plane * N;
+        for (int k = tid; k < A.n_add; k += 256) {
+            const long long cell = __ldg(A.src_cell + k);
+            if (cell < 0 || cell >= n_cells) {
+                if (fb == 0) flag_status(A.status, kStatusBounds);
+                continue;
+            }
+            const unsigned z = (unsigned)cell / (unsigned)plane, at = (unsigned)cell - z * (unsigned)plane;
+            if (at >= i0 && at < i0 + 256 && (int)z >= z0 && (int)z < z1) atomicAdd(A.Cout + cell, __ldg(A.src_emit + k));
+        }
+    }
 }
 
 // Point sources: C'[cell_k] += e_k (atomic, so duplicate cells accumulate).
@@ -287,6 +386,60 @@ int sm_count()
 
 }  // namespace
 
+// One launch of step_any: the field, the cones with `cones`, and the sources where the caller can be told.
+static cudaError_t launch_any(Sim &s, const float *Cin, float *Cout, bool cones, bool *sources_done)
+{
+    const FieldDesc &f = s.fd;
+    AnyArgs A{};
+    A.f = f;
+    A.c = s.cd;
+    A.Cin = Cin;
+    A.Cout = Cout;
+    A.M = s.src_map;
+    const size_t plane = f.dim == 3 ? (size_t)f.nx * f.ny : (size_t)f.nx;
+    const int N = f.dim == 3 ? f.nz : f.ny;
+    A.plane_blocks = (unsigned)((plane + 255) / 256);
+    // as many blocks as the SMs hold (8 each) when the march is long enough to be cut
+    long long chunks = std::max(1LL, std::min<long long>(N, 8LL * sm_count() / A.plane_blocks));
+    A.chunk = (int)((N + chunks - 1) / chunks);
+    chunks = (N + A.chunk - 1) / A.chunk;
+    A.step = (uint32_t)s.cone_step;
+    A.n = cones ? s.n_axons : 0;
+    A.cone_blocks = (unsigned)((A.n + kAnyCones - 1) / kAnyCones);
+    A.pos = s.pos;
+    A.dir = s.dir;
+    A.active = s.active;
+    A.src_xyz = s.src_xyz();
+    A.n_stop = s.cd.stop_r2 >= 0.0f ? s.n_src : 0;
+    A.counter = s.cone_counter();
+    A.src_cell = s.src_cell;
+    A.src_emit = s.src_emit;
+    A.n_add = sources_done && s.n_src <= kAnySources ? s.n_src : 0;
+    if (sources_done) *sources_done = A.n_add == s.n_src;
+    A.status = s.status();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(A.cone_blocks + A.plane_blocks * chunks));
+    cfg.blockDim = dim3(256);
+    cfg.stream = s.stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const bool map = s.src_map != nullptr;
+    if (f.dim == 3) return map ? cudaLaunchKernelEx(&cfg, step_any<3, true>, A) : cudaLaunchKernelEx(&cfg, step_any<3, false>, A);
+    return map ? cudaLaunchKernelEx(&cfg, step_any<2, true>, A) : cudaLaunchKernelEx(&cfg, step_any<2, false>, A);
+}
+
+cudaError_t launch_step_any(Sim &s, const float *Cin, float *Cout, bool *sources_done)
+{
+    timing_begin(s);
+    const cudaError_t e = launch_any(s, Cin, Cout, true, sources_done);
+    timing_end(s);
+    s.launches++;
+    return e;
+}
+
 cudaError_t launch_field_step(Sim &s, const float *Cin, float *Cout, bool *sources_done)
 {
     const FieldDesc &f = s.fd;
@@ -331,11 +484,8 @@ cudaError_t launch_field_step(Sim &s, const float *Cin, float *Cout, bool *sourc
         if (map) field3d_vec4<true, BY><<<grid, block, 0, s.stream>>>(f, Cin, Cout, s.src_map, zchunk, s.status());
         else field3d_vec4<false, BY><<<grid, block, 0, s.stream>>>(f, Cin, Cout, nullptr, zchunk, s.status());
     } else {
-        const size_t n = (size_t)f.nx * f.ny * f.nz;
-        size_t blocks = (n + 255) / 256;
-        if (blocks > (size_t)sm_count() * 64) blocks = (size_t)sm_count() * 64;
-        if (map) field_scalar<true><<<(unsigned)blocks, 256, 0, s.stream>>>(f, Cin, Cout, s.src_map, s.status());
-        else field_scalar<false><<<(unsigned)blocks, 256, 0, s.stream>>>(f, Cin, Cout, nullptr, s.status());
+        const cudaError_t e = launch_any(s, Cin, Cout, false, nullptr);
+        if (e != cudaSuccess) return e;
     }
     timing_end(s);
     s.launches++;

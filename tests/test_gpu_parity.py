@@ -479,3 +479,25 @@ def test_maximum_grid_one_step_on_sampled_windows(cue, dim, offset):
     sim.close()
     del sim, f0, out
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("dim,nx,ny,nz,n,map_", [(3, 33, 9, 3, 200, False), (3, 65, 17, 40, 300, True), (3, 31, 8, 5, 0, False),
+                                                 (3, 129, 97, 65, 5000, False), (2, 101, 99, 1, 257, False),
+                                                 (2, 5, 3, 1, 4, True), (2, 2049, 2051, 1, 500, False)])
+def test_one_launch_steps_of_any_row_length_equal_separate_launches(cue, dim, nx, ny, nz, n, map_):
+    """AUTO steps rows that are not whole float4 groups (and fit no tile engine) in one launch: cones, field and
+    sources; PLAIN takes three.  The whole state agrees bit for bit, odd tiles, map and stops included."""
+    w = W.make("any", dim, nx, ny, nz, dt=0.15 if dim == 3 else 0.2, n_src=5, emit=(0.5, 2.0), n_axons=n, C0="smooth",
+               seed=nx, stop_radius=2.0, src_map="random" if map_ else False)
+    a = cue.Simulation(w, path=cue.CUE_PATH_PLAIN)
+    b = cue.Simulation(w)
+    l0 = b.launches()
+    for s in (a, b):
+        s.sim_run(6)
+        s.check()
+    assert b.last_path() == cue.CUE_PATH_PLAIN and b.launches() - l0 == 6
+    for x, y in zip(a.snapshot(), b.snapshot()):
+        assert np.array_equal(x, y)
+    assert a.cone_updates() == b.cone_updates()
+    a.close()
+    b.close()
