@@ -18,9 +18,11 @@
 // checkpoint storing every step (one persistent launch on 2D grids with
 // nx % 4 == 0, else a cone and a field launch per step).  With ckpt_every >=
 // nsteps the whole run is stored once and nothing is recomputed.  Each segment
-// is then walked backwards: one persistent cooperative launch per segment (adj_persist_kernel:
+// is then walked backwards: one launch that linearises every cone step (adj_linear_kernel)
+// and one persistent cooperative launch per segment (adj_persist_kernel:
 // field warps advance the adjoint field, cone warps scatter the cone adjoint,
-// one bounded grid barrier per step), or, where that launch does not apply, a
+// one bounded grid barrier per step; more pairs of launches where the
+// linearisations of a segment exceed their buffer), or, where that launch does not apply, a
 // field launch and a cone launch per step.
 //
 // Precision: the adjoint field is double-float (two FP32 planes carried with
@@ -474,10 +476,22 @@ __device__ __forceinline__ void cone_adjoint3(const FieldDesc &f, const ConeDesc
     for (int i = 0; i < DIM; ++i) pbar[i] = pb[i];
 }
 
-__device__ __forceinline__ void cone_adjoint2(const FieldDesc &f, const ConeDesc &c, double inv_hd,
+// One 2D cone step's linearisation: everything its reverse mode needs that does not depend on what comes back
+// from the later steps.
+constexpr unsigned kConeHasG = 1, kConeHasV = 2, kConeClamp0 = 4, kConeClamp1 = 8;
+struct Cone2 {
+    int lo[2];                        // its cell
+    unsigned flags;
+    double dn[2], vinv, ghat[2], ginv;
+    double gx[4], gy[4];              // corner gradients (00, 10, 01, 11)
+    double fr[2];                     // weights within the cell
+};
+
+__device__ __forceinline__ Cone2 cone_linear2(const FieldDesc &f, const ConeDesc &c, double inv_hd,
                                               const float *__restrict__ C, uint32_t axon, uint32_t step,
-                                              const float *p, const float *d, double *pbar, double *dbar, float *mu)
+                                              const float *p, const float *d)
 {
+    Cone2 L;
     const size_t sy = f.nx;
     auto ld = [&](int i, int j, int) { return __ldg(C + (size_t)i + sy * j); };
     // the forward step in FP32, for its decisions (gradient threshold, blend
@@ -516,32 +530,57 @@ __device__ __forceinline__ void cone_adjoint2(const FieldDesc &f, const ConeDesc
     // in FP64 from the FP32 node values and position (inv_hd = 1/h in FP64);
     // the per-cone work is small next to the field's
     const double i2h = (double)c.inv2h;
-    const double frx = (double)p[0] * inv_hd - (double)lo[0], fry = (double)p[1] * inv_hd - (double)lo[1];
-    const double wx0 = 1.0 - frx, wx1 = frx, wy0 = 1.0 - fry, wy1 = fry;
+    L.fr[0] = (double)p[0] * inv_hd - (double)lo[0];
+    L.fr[1] = (double)p[1] * inv_hd - (double)lo[1];
+    const double wx0 = 1.0 - L.fr[0], wx1 = L.fr[0], wy0 = 1.0 - L.fr[1], wy1 = L.fr[1];
     const double w00 = wx0 * wy0, w10 = wx1 * wy0, w01 = wx0 * wy1, w11 = wx1 * wy1;
-    const double gx00 = ((double)v[2] - v[0]) * i2h, gx10 = ((double)v[3] - v[1]) * i2h;
-    const double gx01 = ((double)v[6] - v[4]) * i2h, gx11 = ((double)v[7] - v[5]) * i2h;
-    const double gy00 = ((double)v[5] - v[8]) * i2h, gy10 = ((double)v[6] - v[9]) * i2h;
-    const double gy01 = ((double)v[10] - v[1]) * i2h, gy11 = ((double)v[11] - v[2]) * i2h;
-    const double gd[2] = {w00 * gx00 + w10 * gx10 + w01 * gx01 + w11 * gx11,
-                          w00 * gy00 + w10 * gy10 + w01 * gy01 + w11 * gy11};
-    double ghat[2] = {0.0, 0.0}, ginvd = 0.0;
+    L.gx[0] = ((double)v[2] - v[0]) * i2h;
+    L.gx[1] = ((double)v[3] - v[1]) * i2h;
+    L.gx[2] = ((double)v[6] - v[4]) * i2h;
+    L.gx[3] = ((double)v[7] - v[5]) * i2h;
+    L.gy[0] = ((double)v[5] - v[8]) * i2h;
+    L.gy[1] = ((double)v[6] - v[9]) * i2h;
+    L.gy[2] = ((double)v[10] - v[1]) * i2h;
+    L.gy[3] = ((double)v[11] - v[2]) * i2h;
+    const double gd[2] = {w00 * L.gx[0] + w10 * L.gx[1] + w01 * L.gx[2] + w11 * L.gx[3],
+                          w00 * L.gy[0] + w10 * L.gy[1] + w01 * L.gy[2] + w11 * L.gy[3]};
+    L.ginv = L.ghat[0] = L.ghat[1] = 0.0;
     if (has_g) {
-        ginvd = rsqrt_d(gd[0] * gd[0] + gd[1] * gd[1]);
-        ghat[0] = gd[0] * ginvd;
-        ghat[1] = gd[1] * ginvd;
+        L.ginv = rsqrt_d(gd[0] * gd[0] + gd[1] * gd[1]);
+        L.ghat[0] = gd[0] * L.ginv;
+        L.ghat[1] = gd[1] * L.ginv;
     }
-    double vd[2], dn[2], vinvd = 0.0;
+    double vd[2];
+    L.vinv = 0.0;
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-        vd[i] = (double)c.w_prev * (double)d[i] + (double)c.w_grad * ghat[i] + (double)c.w_noise * (double)xi[i];
-    if (has_v) vinvd = rsqrt_d(vd[0] * vd[0] + vd[1] * vd[1]);
+        vd[i] = (double)c.w_prev * (double)d[i] + (double)c.w_grad * L.ghat[i] + (double)c.w_noise * (double)xi[i];
+    if (has_v) L.vinv = rsqrt_d(vd[0] * vd[0] + vd[1] * vd[1]);
 #pragma unroll
-    for (int i = 0; i < 2; ++i) dn[i] = has_v ? vd[i] * vinvd : (double)d[i];
+    for (int i = 0; i < 2; ++i) L.dn[i] = has_v ? vd[i] * L.vinv : (double)d[i];
+    L.lo[0] = lo[0];
+    L.lo[1] = lo[1];
+    L.flags = (has_g ? kConeHasG : 0) | (has_v ? kConeHasV : 0) | (clamped[0] ? kConeClamp0 : 0) |
+              (clamped[1] ? kConeClamp1 : 0);
+    return L;
+}
+
+// Back through that step: (pbar, dbar) of its end become those of its start, and its part of the adjoint field goes
+// into mu.
+__device__ __forceinline__ void cone_back2(const FieldDesc &f, const ConeDesc &c, double inv_hd, const Cone2 &L,
+                                           double *pbar, double *dbar, float *mu)
+{
+    const size_t sy = f.nx;
+    const int *lo = L.lo;
+    const double *dn = L.dn, *ghat = L.ghat;
+    const bool has_g = L.flags & kConeHasG, has_v = L.flags & kConeHasV;
+    const double i2h = (double)c.inv2h;
+    const double wx0 = 1.0 - L.fr[0], wx1 = L.fr[0], wy0 = 1.0 - L.fr[1], wy1 = L.fr[1];
+    const double w00 = wx0 * wy0, w10 = wx1 * wy0, w01 = wx0 * wy1, w11 = wx1 * wy1;
     double qbar[2], dnbar[2];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-        qbar[i] = clamped[i] ? 0.0 : pbar[i];
+        qbar[i] = (L.flags & (kConeClamp0 << i)) ? 0.0 : pbar[i];
         dnbar[i] = (double)c.step_len * qbar[i] + dbar[i];
     }
     double vbar[2];
@@ -549,7 +588,7 @@ __device__ __forceinline__ void cone_adjoint2(const FieldDesc &f, const ConeDesc
         const double dot = dn[0] * dnbar[0] + dn[1] * dnbar[1];
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            vbar[i] = (dnbar[i] - dn[i] * dot) * vinvd;
+            vbar[i] = (dnbar[i] - dn[i] * dot) * L.vinv;
             dbar[i] = (double)c.w_prev * vbar[i];
         }
     } else {
@@ -564,12 +603,12 @@ __device__ __forceinline__ void cone_adjoint2(const FieldDesc &f, const ConeDesc
         const double wg = (double)c.w_grad;
         const double dot = ghat[0] * (wg * vbar[0]) + ghat[1] * (wg * vbar[1]);
 #pragma unroll
-        for (int i = 0; i < 2; ++i) gbar[i] = (wg * vbar[i] - ghat[i] * dot) * ginvd;
+        for (int i = 0; i < 2; ++i) gbar[i] = (wg * vbar[i] - ghat[i] * dot) * L.ginv;
     }
     // position: g(p) = sum_c w_c(p) G_c (corner (a, b) = node (x_a, y_b)), dw/dp
     // from the bilinear weights
-    const double s00 = gbar[0] * gx00 + gbar[1] * gy00, s10 = gbar[0] * gx10 + gbar[1] * gy10;
-    const double s01 = gbar[0] * gx01 + gbar[1] * gy01, s11 = gbar[0] * gx11 + gbar[1] * gy11;
+    const double s00 = gbar[0] * L.gx[0] + gbar[1] * L.gy[0], s10 = gbar[0] * L.gx[1] + gbar[1] * L.gy[1];
+    const double s01 = gbar[0] * L.gx[2] + gbar[1] * L.gy[2], s11 = gbar[0] * L.gx[3] + gbar[1] * L.gy[3];
     const double ih = inv_hd;
     pbar[0] = ih * (wy0 * (s10 - s00) + wy1 * (s11 - s01)) + qbar[0];
     pbar[1] = ih * (wx0 * (s01 - s00) + wx1 * (s11 - s10)) + qbar[1];
@@ -605,6 +644,13 @@ __device__ __forceinline__ void cone_adjoint2(const FieldDesc &f, const ConeDesc
     }
 }
 
+__device__ __forceinline__ void cone_adjoint2(const FieldDesc &f, const ConeDesc &c, double inv_hd,
+                                              const float *__restrict__ C, uint32_t axon, uint32_t step,
+                                              const float *p, const float *d, double *pbar, double *dbar, float *mu)
+{
+    cone_back2(f, c, inv_hd, cone_linear2(f, c, inv_hd, C, axon, step, p, d), pbar, dbar, mu);
+}
+
 // ---------------------------------------------------------------- persistent backward
 // The cone adjoint never reads the adjoint field: going back through step m,
 //   mu^m = A mu^{m+1} + X^m,   X^m = the cones' scatter at step m.
@@ -628,6 +674,10 @@ struct AdjP {
     size_t cells, cone_n;
     float *Y[2];
     float *X[3];
+    double *lin;                  // linearisations: kLinD planes of n (padded) doubles a step,
+    int4 *lin_i;                  // and a plane of (cell, flags)
+    size_t lin_n;
+    int lin_m0;                   // the first stored step
     float *Sseg;                  // nullable
     double *part;                 // per-block (dD, dlambda) slots
     double *de;                   // per-source sums
@@ -646,6 +696,35 @@ struct AdjRow {
     float4 yh, yl, xh, xl;
     float e[4];                  // lane 0: column x - 1, lane 31: column x + 4 (yh, yl, xh, xl)
 };
+
+constexpr int kLinD = 16;
+
+// The linearisations of steps m0 .. m0 + gridDim.y - 1 of a segment.
+//
+// Formed by the warp that steps the cones back, they were the longer part of a serial chain in every backward step
+// (FP64 at GB300's low rate, behind a gather from L2), which no other warp could shorten.  They do not depend on the
+// later steps, so they are formed for many steps at once, every SM busy (0.75 us a step with 4,096 cones, FP64-bound;
+// 0.1 with 64), and the backward launch loads 144 bytes a cone and keeps the part that is a recursion.  The whole
+// gradient, us a step of the run: 128^2 with 64 cones 11.65 -> 9.26, 512^2 with 8 12.0 -> 9.5, with 4,096 26.6 -> 24.7,
+// 1024^2 with 4,096 and a map 21.1 -> 20.4 (there the field's instructions bound the step).
+__global__ void __launch_bounds__(128) adj_linear_kernel(AdjP A, uint32_t g0)
+{
+    const int a = blockIdx.x * 128 + threadIdx.x, j = blockIdx.y, m = A.lin_m0 + j;
+    if (a >= A.n || !A.active[a]) return;
+    const float *Pm = A.segP + 2 * A.cone_n * m;
+    float p[2], d[2];
+    for (int i = 0; i < 2; ++i) {
+        p[i] = __ldg(Pm + (size_t)i * A.n + a);
+        d[i] = __ldg(Pm + A.cone_n + (size_t)i * A.n + a);
+    }
+    const Cone2 L = cone_linear2(A.f, A.c, A.inv_h64, A.segC + A.cells * m, (uint32_t)a, g0 + (uint32_t)m, p, d);
+    const double v[kLinD] = {L.dn[0], L.dn[1], L.vinv,  L.ghat[0], L.ghat[1], L.ginv,  L.gx[0], L.gx[1],
+                             L.gx[2], L.gx[3], L.gy[0], L.gy[1],   L.gy[2],   L.gy[3], L.fr[0], L.fr[1]};
+    double *o = A.lin + (size_t)j * kLinD * A.lin_n + a;
+#pragma unroll
+    for (int q = 0; q < kLinD; ++q) o[q * A.lin_n] = v[q];
+    A.lin_i[(size_t)j * A.lin_n + a] = make_int4(L.lo[0], L.lo[1], (int)L.flags, 0);
+}
 
 __device__ __forceinline__ void adj_row_load(const AdjP &A, const float *Yin, const float *Xin, int y, int x4,
                                              bool xin, bool has_l, bool has_r, AdjRow &R)
@@ -762,13 +841,13 @@ __device__ __forceinline__ void adj_rows(const AdjP &A, const float *Yin, const 
     }
 }
 
-__global__ void __launch_bounds__(256, 2) adj_persist_kernel(AdjP A, int len, uint32_t g0, PBar *bar,
+__global__ void __launch_bounds__(256, 2) adj_persist_kernel(AdjP A, int m1, uint32_t g0, PBar *bar,
                                                              unsigned expected, long long limit, unsigned *status)
 {
     // each thread's dD and dlambda products, summed over the segment's steps in
     // compensated FP32 (two_sum: hi + lo), reduced over the block once at the end
     DF sD{0.f, 0.f}, sL{0.f, 0.f};
-    for (int m = len - 1; m >= 0; --m) {
+    for (int m = m1 - 1; m >= A.lin_m0; --m) {
         const uint32_t g = g0 + (uint32_t)m;              // global step index
         const float *Yin = A.Y[(g + 1) & 1];
         float *Yout = A.Y[g & 1];
@@ -776,7 +855,6 @@ __global__ void __launch_bounds__(256, 2) adj_persist_kernel(AdjP A, int len, ui
         float *Xout = A.X[g % 3];
         float *Xz = A.X[(g + 2) % 3];
         const float *Cm = A.segC + A.cells * m;
-        const float *Pm = A.segP + 2 * A.cone_n * m;
         if (blockIdx.x == 0)                              // de_k += mu^{m+1}[cell_k]
             for (int k = threadIdx.x; k < A.n_src; k += blockDim.x) {
                 const long long c = A.src_cell[k];
@@ -797,15 +875,18 @@ __global__ void __launch_bounds__(256, 2) adj_persist_kernel(AdjP A, int len, ui
         for (int chunk = bid; cone_warp && chunk < A.n_chunks; chunk += A.n_cone_warps) {
             const int a = chunk * 32 + (threadIdx.x & 31);
             if (a < A.n && A.active[a]) {
-                float p[2], d[2];
-                double pb[2], db[2];
+                double pb[2], db[2], v[kLinD];
                 for (int i = 0; i < 2; ++i) {
-                    p[i] = __ldg(Pm + (size_t)i * A.n + a);
-                    d[i] = __ldg(Pm + A.cone_n + (size_t)i * A.n + a);
                     pb[i] = __ldcg(A.pbar + (size_t)i * A.n + a);
                     db[i] = __ldcg(A.dbar + (size_t)i * A.n + a);
                 }
-                cone_adjoint2(A.f, A.c, A.inv_h64, Cm, (uint32_t)a, g, p, d, pb, db, Xout);
+                const double *lin = A.lin + (size_t)(m - A.lin_m0) * kLinD * A.lin_n + a;
+#pragma unroll
+                for (int q = 0; q < kLinD; ++q) v[q] = __ldg(lin + q * A.lin_n);
+                const int4 li = __ldg(A.lin_i + (size_t)(m - A.lin_m0) * A.lin_n + a);
+                const Cone2 L{{li.x, li.y}, (unsigned)li.z, {v[0], v[1]}, v[2], {v[3], v[4]}, v[5],
+                              {v[6], v[7], v[8], v[9]}, {v[10], v[11], v[12], v[13]}, {v[14], v[15]}};
+                cone_back2(A.f, A.c, A.inv_h64, L, pb, db, Xout);
                 for (int i = 0; i < 2; ++i) {
                     A.pbar[(size_t)i * A.n + a] = pb[i];
                     A.dbar[(size_t)i * A.n + a] = db[i];
@@ -948,7 +1029,7 @@ __global__ void __launch_bounds__(256) adj_finalize_kernel(FieldDesc f, int n_ax
 }
 
 struct AdjLayout {
-    size_t ckpt_c, ckpt_p, seg_c, seg_p, mu, Sseg, S, pbar, acc, part, bar, total;
+    size_t ckpt_c, ckpt_p, seg_c, seg_p, mu, Sseg, S, pbar, acc, part, bar, lin, lin_i, total;
     int n_part;
     int nseg;
 };
@@ -1000,6 +1081,15 @@ AdjFieldShape adj_field_shape(const cue_params &p)
 
 int adj_field_blocks(const cue_params &p) { return adj_field_shape(p).blocks; }
 
+// Linearisations are kept for as many steps as take 64 MB (half of the L2: the backward launch reads them from there), one
+// at least: 64 steps of 7,281 cones.  A launch over fewer steps costs its start, about 6 us.
+size_t adj_lin_stride(int n_axons) { return ((size_t)n_axons + 31) / 32 * 32; }
+int adj_lin_steps(int n_axons, int len)
+{
+    const size_t bytes = adj_lin_stride(n_axons) * (kLinD * sizeof(double) + sizeof(int4));
+    return (int)std::min<size_t>((size_t)len, std::max<size_t>(1, ((size_t)64 << 20) / std::max<size_t>(bytes, 1)));
+}
+
 AdjLayout adj_layout(const cue_params &p, int n_src, int n_axons, int nsteps, int k)
 {
     AdjLayout L{};
@@ -1031,6 +1121,13 @@ AdjLayout adj_layout(const cue_params &p, int n_src, int n_axons, int nsteps, in
     off += align256(sizeof(double) * 2 * (size_t)L.n_part);
     L.bar = off;                                  // grid barrier of the persistent backward
     off += 256;
+    if (p.dim == 2 && n_axons > 0) {              // cone linearisations of a run of steps
+        const size_t per = adj_lin_stride(n_axons) * (size_t)adj_lin_steps(n_axons, std::min(k, nsteps));
+        L.lin = off;
+        off += align256(sizeof(double) * kLinD * per);
+        L.lin_i = off;
+        off += align256(sizeof(int4) * per);
+    }
     L.total = off;
     return L;
 }
@@ -1197,6 +1294,9 @@ int run_adjoint(Sim &s, const float *targets, int nsteps, int k, void *ws, size_
         A.Y[1] = base + 2 * cells;
         for (int i = 0; i < 3; ++i) A.X[i] = base + (4 + 2 * i) * cells;
         A.Sseg = Sseg;
+        A.lin = reinterpret_cast<double *>(W + L.lin);
+        A.lin_i = reinterpret_cast<int4 *>(W + L.lin_i);
+        A.lin_n = adj_lin_stride(n);
         A.part = part;
         A.de = acc + 2;
         A.ntx = (f.nx / 4 + 31) / 32;
@@ -1226,7 +1326,6 @@ int run_adjoint(Sim &s, const float *targets, int nsteps, int k, void *ws, size_
         if (persist_bw) {
             A.segC = sgC;
             A.segP = sgP;
-            if (!ok(cudaMemsetAsync(W + L.bar, 0, 256, st))) return CUE_ERR_CUDA;
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(bw_grid);
             cfg.blockDim = dim3(256);
@@ -1236,11 +1335,20 @@ int run_adjoint(Sim &s, const float *targets, int nsteps, int k, void *ws, size_
             attr[0].val.cooperative = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            if (!ok(cudaLaunchKernelEx(&cfg, adj_persist_kernel, A, len, (uint32_t)nstart,
-                                       reinterpret_cast<PBar *>(W + L.bar), (unsigned)bw_grid, kPersistSpinLimit,
-                                       s.status())))
-                return CUE_ERR_CUDA;
-            s.launches++;
+            const int run = n > 0 ? adj_lin_steps(n, len) : len;
+            for (int m1 = len; m1 > 0; m1 -= run) {
+                A.lin_m0 = std::max(0, m1 - run);
+                if (n > 0) {
+                    adj_linear_kernel<<<dim3((n + 127) / 128, m1 - A.lin_m0), 128, 0, st>>>(A, (uint32_t)nstart);
+                    s.launches++;
+                }
+                if (!ok(cudaMemsetAsync(W + L.bar, 0, 256, st)) ||
+                    !ok(cudaLaunchKernelEx(&cfg, adj_persist_kernel, A, m1, (uint32_t)nstart,
+                                           reinterpret_cast<PBar *>(W + L.bar), (unsigned)bw_grid, kPersistSpinLimit,
+                                           s.status())))
+                    return CUE_ERR_CUDA;
+                s.launches++;
+            }
         }
         for (int m = len - 1; !persist_bw && m >= 0; --m) {
             const float *Cm = sgC + cells * m, *Pm = sgP + 2 * cone_n * m;

@@ -297,6 +297,37 @@ def test_full_size_persistent_backward_equals_two_launch_backward(cue):
         assert np.abs(x - y).max() <= 1e-4 * scale, key
 
 
+@pytest.mark.parametrize("nx,ny,n_axons,nsteps,k", [
+    (132, 5, 40, 11, 4),          # a second strip one lane wide; fewer rows than warps
+    (4, 3, 3, 7, 7),              # the smallest: every scatter folded at a wall
+    (260, 900, 700, 9, 3),        # three strips, two rows a warp at most
+    (128, 31000, 300, 5, 3),      # a dozen rows a warp
+    (256, 192, 9000, 70, 64),     # more cones than one run of linearisations over the segment holds
+])
+def test_persistent_backward_equals_launches_per_step_at_odd_shapes(cue, nx, ny, n_axons, nsteps, k):
+    """The persistent backward takes the cones' linearisations from a launch before it, for a
+    bounded number of steps, and shares its rows out between warps; the launches per step do
+    neither.  Same states, the same double-float sums in another order: the emission and map
+    gradients agree to ADJ_RTOL of their largest entry.  (dD and dlambda are FP32 products over a
+    smooth field whose large terms cancel; they are held to the FP64 oracle on the identical
+    states below.)"""
+    w = W.make("shape", 2, nx, ny, n_src=2, n_axons=n_axons, C0="smooth", seed=nx + ny, wall_mode=1,
+               src_map="zeros", targets=True)
+    out = []
+    for path in (None, cue.CUE_PATH_PLAIN):
+        sim = cue.Simulation(w) if path is None else cue.Simulation(w, path=path)
+        g = sim.adjoint(w.targets, nsteps, k)
+        sim.check()
+        out.append({key: (None if v is None else v.cpu().numpy()) for key, v in g.items()})
+        sim.close()
+    a, b = out
+    assert a["loss"] == b["loss"]
+    for key in ("dsrc", "dmap"):
+        x, y = a[key].astype(np.float64), b[key].astype(np.float64)
+        scale = max(np.abs(y).max(), 1e-30)
+        assert np.abs(x - y).max() <= ADJ_RTOL * scale, key
+
+
 def test_adjoint_full_horizon_on_the_small_copy_is_reported(cue, record_property):
     """The adjoint workload's 64x64 copy over its full 2,000 steps (checkpoint every 64): the
     GPU gradients, the FP64 oracle's adjoint and FP64 central differences of the oracle's loss
