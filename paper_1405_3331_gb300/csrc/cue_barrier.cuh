@@ -13,7 +13,9 @@ namespace cue {
 // orders before it), and the barrier is passed once the counter reaches the
 // next multiple of `expected`: the last arrival needs no second write, and
 // the others poll with acquire loads, a bounded number of times.  Returns
-// false when the launch is aborting.
+// false when the launch is aborting: the flag is looked at every 32 polls
+// only, since each look is a trip to L2 that the wait's end would be noticed
+// after (a block that arrives later waits for one that has left, and looks).
 __device__ __forceinline__ unsigned long long atom_add_acq_rel(unsigned long long *p, unsigned long long v)
 {
     unsigned long long old;
@@ -34,24 +36,22 @@ __device__ __forceinline__ bool grid_barrier(PBar *bar, unsigned expected, long 
     __syncthreads();
     if (threadIdx.x == 0) {
         volatile int *vabort = &bar->abort;
-        int ok = *vabort ? 0 : 1;
-        if (ok) {
-            const unsigned long long ticket = atom_add_acq_rel(&bar->count, 1ull);
-            const unsigned long long target = (ticket / expected + 1ull) * expected;
-            long long it = 0;
-            while (ld_acquire(&bar->count) < target) {
-                if (*vabort) {
-                    ok = 0;
-                    break;
-                }
-                if (++it > limit) {
-                    flag_status(status, kStatusTimeout);
-                    atomicExch(&bar->abort, 1);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(32);
+        int ok = 1;
+        const unsigned long long ticket = atom_add_acq_rel(&bar->count, 1ull);
+        const unsigned long long target = (ticket / expected + 1ull) * expected;
+        long long it = 0;
+        while (ld_acquire(&bar->count) < target) {
+            if ((++it & 31) == 0 && *vabort) {
+                ok = 0;
+                break;
             }
+            if (it > limit) {
+                flag_status(status, kStatusTimeout);
+                atomicExch(&bar->abort, 1);
+                ok = 0;
+                break;
+            }
+            __nanosleep(32);
         }
         s_ok = ok;
     }
