@@ -865,6 +865,9 @@ __device__ __forceinline__ unsigned cone_loop(const TileArgs &A, const Tile &T, 
                 }
             }
             if (!ok) *s_fail = 1;
+            // every round's first step finds its ticket at zero: a crowded step clears the next step's only, so
+            // its round leaves its last step's as it was
+            if (lane < 2) s_ticket[lane] = 0;
         }
         block_sync();
         if (*s_fail) break;

@@ -130,6 +130,54 @@ def test_adjoint_states_on_tiles_are_the_plain_path_s(cue, nx, ny):
         assert np.array_equal(got[0][k].cpu().numpy(), got[1][k].cpu().numpy()), k
 
 
+# A strip of one tile row whose tile borders in x are known: W = 128 loaded columns, a halo of K + 1 nodes and the drift
+# of K - 1 steps of 0.05 (one node), rounded up to whole float4 groups.
+FLIP_TILES = range(3, 79, 5)
+
+
+def _flip_case(depth, rate_map=False):
+    """Tiles that hold 124 cones in their middle and 10 around their border, walking at random: their number
+    rises above 128 (the cones a tile steps from registers), falls to 128 or below and rises again, for rounds of any number."""
+    halo = (depth + 1 + (depth > 1) + 3) // 4 * 4
+    first, inner = 128 - halo, 128 - 2 * halo
+    n = 134 * len(FLIP_TILES)
+    w = W.make("flip", 2, 9600, 16, n_src=9, emit=(0.5, 2.0), n_axons=n, C0="smooth", seed=40 + depth, wall_mode=1,
+               src_map="random" if rate_map else False, targets=True, w=(0.0, 0.1, 1.0), step_len=0.05)
+    rng = np.random.default_rng(depth)
+    for i, k in enumerate(FLIP_TILES):
+        left = first + (k - 1) * inner
+        x = np.concatenate([left + rng.uniform(20, inner - 20, 124), left + rng.uniform(-0.2, 0.2, 10)])
+        w.pos[0, 134 * i : 134 * (i + 1)] = x
+        w.pos[1, 134 * i : 134 * (i + 1)] = rng.uniform(2, 13, 134)
+    tile = lambda x: np.where(x < first, 0, 1 + (np.floor(x) - first) // inner)
+    return w, lambda x: np.array([(tile(x) == k).sum() for k in FLIP_TILES])
+
+
+def _returns(crowds):
+    """How often a tile is crowded again after an odd number of rounds in which it was not."""
+    found = 0
+    for c in np.array(crowds).T > 128:
+        at = np.flatnonzero(c)
+        found += int(((np.diff(at) > 1) & (np.diff(at) % 2 == 0)).sum())
+    return found
+
+
+@pytest.mark.parametrize("depth,rate_map", [(1, False), (3, False), (5, True), (7, False), (8, False)])
+def test_stored_states_of_tiles_that_are_crowded_now_and_then(cue, depth, rate_map):
+    w, crowd = _flip_case(depth, rate_map)
+    steps, got = max(26 * depth, 100), []
+    for path in (cue.CUE_PATH_PLAIN, cue.CUE_PATH_AUTO):
+        sim = cue.Simulation(w, path=path)
+        sim.set_option(cue.CUE_OPT_TEMPORAL_DEPTH, depth)
+        got.append(sim.adjoint(w.targets, steps, steps, trace=True))
+        sim.check()
+        sim.close()
+    plain, tiles = ({k: g[k].cpu().numpy() for k in ("trace_cone", "trace_C", "loss")} for g in got)
+    assert _returns([crowd(plain["trace_cone"][s, 0, 0]) for s in range(0, steps, depth)]) > 0
+    for k in plain:
+        assert np.array_equal(plain[k], tiles[k]), k
+
+
 def test_device_side_problems_are_reported(cue):
     """Non-finite input is reported; sources outside the grid are skipped and reported."""
     w = _case("512x300")
