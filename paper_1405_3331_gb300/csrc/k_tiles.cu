@@ -48,6 +48,17 @@
 // two half-sized tiles per SM (more border: 60% slower), 6 or 8 cone warps (10% slower with few cones a tile,
 // 20% faster with hundreds), the cone warps on a scheduler of their own (the field's three then bound the step).
 //
+// The caller's arrays are read once, at the start: a block loads its tile and looks through all
+// cones for those inside its interior, then raises its flag.  Until a block knows its neighbours' flags it
+// writes neither field nor cone state: a neighbour that came later would find a cone that had
+// moved into its interior, take it for its own and step it again.  What goes out in the first
+// round (a run of one round, cones that stop, cones past a full list) waits for them where it is written; the
+// arrivals warp looks for them in the first exchange, whose last barrier frees every later round.
+// The neighbours are enough: no one farther away takes a cone for its own, whatever mix of an old and a new coordinate
+// it reads, because a block in its round r has had the exchanges of r rounds, so blocks within r tiles have
+// loaded, and a cone it writes came from r tiles away at most and is now one tile away at most.
+// (Trajectory mode reads slot 0 and writes the later ones, and its cones do not stop.)
+//
 // Arithmetic per node and per cone is the plain path's (update4 = node_update2,
 // the map as fma(dt, M, C'), sources added after it in index order; cone_step_rule),
 // bit for bit.  Every wait is bounded, as in cue_barrier.cuh: past the limit the
@@ -205,6 +216,22 @@ __device__ __forceinline__ bool wait_neighbours(const TileArgs &A, int tx, int t
         while (ok && (int)(ld_acquire_u32(flag) - want) < 0) ok = keep_waiting(it, A.limit, A.abort, A.base, A.status);
     }
     return __all_sync(kFull, ok);
+}
+
+// The same for one lane, in the rare places where a lane alone has cone state to write in the first round; a wait
+// given up also ends the block's run.
+__device__ __noinline__ bool neighbours_loaded(const TileArgs &A, int tx, int ty, volatile int *s_fail)
+{
+    bool ok = true;
+    long long it = 0;
+    for (int q = 0; q < 9 && ok; ++q) {
+        const int nx = tx + q % 3 - 1, ny = ty + q / 3 - 1;
+        if (q == 4 || nx < 0 || nx >= A.gx || ny < 0 || ny >= A.gy) continue;
+        const unsigned *flag = A.flags + kTlFlagWords * (ny * A.gx + nx);
+        while (ok && (int)(ld_acquire_u32(flag) - A.base) < 0) ok = keep_waiting(it, A.limit, A.abort, A.base, A.status);
+    }
+    if (!ok) *s_fail = 1;
+    return ok;
 }
 
 // Cone state after s steps of this launch: the caller's arrays, or the trajectory's slot.
@@ -583,9 +610,12 @@ __device__ __forceinline__ unsigned field_loop(const TileArgs &A, const Tile &T,
         const unsigned tag = A.base + (unsigned)rd;
         if (m + n_ovf > kTlOwn) {                       // a crowded tile: this warp helps with the cones
             int *ovf = inbox_of(A, rd & 1, T.t) + s_list[1];
+            // (its cones from global memory are written in every step)
+            const bool may = TRAJ || rd > 0 || wait_neighbours(A, T.tx, T.ty, A.base);
+            if (!may) *s_fail = 1;
             for (int s = done; s < done + kr; ++s) {
                 field_step_any<MAP, TRAJ, VEC>(A, T, r0, r1, s, L.own, src);
-                live += crowd_cones<TRAJ>(A, T, T.S + (s & 1 ? T.R * kTlW : 0), s, rd & 1, m, n_ovf, ovf, s_ticket + (s & 1));
+                if (may) live += crowd_cones<TRAJ>(A, T, T.S + (s & 1 ? T.R * kTlW : 0), s, rd & 1, m, n_ovf, ovf, s_ticket + (s & 1));
                 if (s + 1 < done + kr || !last) block_sync();   // (before the last barrier the cone warps place the crowd)
             }
         } else {
@@ -652,9 +682,12 @@ __device__ __forceinline__ unsigned cone_loop(const TileArgs &A, const Tile &T, 
                     xi[1] = s_xi[(s & 1) * 2 * kTlHelped + kTlHelped + slot];
                 }
                 const bool alive = tile_cone_step(A, T, in, xi, p, d, bits);
-                if (TRAJ || !alive) put_cone<TRAJ>(A, s + 1, a, p, d);
+                if (TRAJ) put_cone<TRAJ>(A, s + 1, a, p, d);
                 if (!alive) {
-                    A.active[a] = 0;
+                    if (TRAJ || rd > 0 || neighbours_loaded(A, T.tx, T.ty, s_fail)) {
+                        if (!TRAJ) put_cone<false>(A, 0, a, p, d);
+                        A.active[a] = 0;
+                    }
                     a = -1;
                 } else if (!helped && j + 1 < kr) {
                     cone_noise<2>(A.c.key0, A.c.key1, (uint32_t)a, A.step0 + (uint32_t)(s + 1), xi);
@@ -668,10 +701,12 @@ __device__ __forceinline__ unsigned cone_loop(const TileArgs &A, const Tile &T, 
             }
         };
         if (m + n_ovf > kTlOwn) {                       // a crowded tile
+            const bool may = TRAJ || rd > 0 || wait_neighbours(A, T.tx, T.ty, A.base);
+            if (!may) *s_fail = 1;
             for (int j = 0; j < kr; ++j) {
                 const int s = done + j;
                 own_step(j);
-                live += crowd_cones<TRAJ>(A, T, T.S + (s & 1 ? R * kTlW : 0), s, lb, m, n_ovf, ovf, s_ticket + (s & 1));
+                if (may) live += crowd_cones<TRAJ>(A, T, T.S + (s & 1 ? R * kTlW : 0), s, lb, m, n_ovf, ovf, s_ticket + (s & 1));
                 if (cw == 0 && lane == 0) s_ticket[(s & 1) ^ 1] = 0;
                 if (j + 1 < kr) block_sync();
             }
@@ -685,9 +720,11 @@ __device__ __forceinline__ unsigned cone_loop(const TileArgs &A, const Tile &T, 
         const bool final = rd + 1 == nrounds;
         if (final) {
             if (!TRAJ) {
-                if (a >= 0) put_cone<false>(A, 0, a, p, d);
+                const bool may = rd > 0 || n == 0 || wait_neighbours(A, T.tx, T.ty, A.base);
+                if (!may) *s_fail = 1;
+                if (may && a >= 0) put_cone<false>(A, 0, a, p, d);
                 block_sync();                           // the other warps are done with the list
-                for (int i = kTlOwn + slot; i < m; i += kTlOwn) {
+                for (int i = kTlOwn + slot; may && i < m; i += kTlOwn) {
                     const int c = T.l_id[lb * cap + i];
                     const float cp[2] = {T.st(cap, lb, 0, i), T.st(cap, lb, 1, i)}, cd[2] = {T.st(cap, lb, 2, i), T.st(cap, lb, 3, i)};
                     if (c >= 0) put_cone<false>(A, 0, c, cp, cd);
@@ -732,7 +769,7 @@ __device__ __forceinline__ unsigned cone_loop(const TileArgs &A, const Tile &T, 
                 }
             }
             extra = true;
-            if (!TRAJ && !in_arrays) put_cone<false>(A, 0, c, cp, cd);
+            if (!TRAJ && !in_arrays && (rd > 0 || neighbours_loaded(A, T.tx, T.ty, s_fail))) put_cone<false>(A, 0, c, cp, cd);
             const int to = T.t + dy * A.gx + dx;
             inbox_of(A, np, to)[atomicAdd(A.cnt_cur + np * kTilesMax + to, 1)] = c;
         };
@@ -777,7 +814,8 @@ __device__ __forceinline__ unsigned cone_loop(const TileArgs &A, const Tile &T, 
         block_sync();                                   // the round's last barrier
         if (cw == kTlConeWarps - 1) {
             // ---- arrivals: the number from each neighbour, then its cones, spread over the lanes
-            bool ok = true;
+            // (in the first round, also: the neighbours have loaded, so this block may write from here on)
+            bool ok = TRAJ || rd > 0 || wait_neighbours(A, T.tx, T.ty, A.base);
             if (n > 0) {
                 long long it = 0;
                 int c = 0;
@@ -1015,7 +1053,7 @@ __global__ void __launch_bounds__(kTlThreads, 1) tiles_kernel(const __grid_const
     __syncthreads();
     const int nrounds = (A.nsteps + A.K - 1) / A.K;
     if (tid == 0) {
-        if (!TRAJ && nrounds == 1) st_release_u32(A.flags + kTlFlagWords * T.t, A.base);   // the tile is loaded
+        if (!TRAJ) st_release_u32(A.flags + kTlFlagWords * T.t, A.base);   // the tile is loaded, its cones are found
         s_list[0] = min(s_push, cap);
         s_list[1] = 0;
         s_list[2] = s_push - min(s_push, cap);
@@ -1048,8 +1086,8 @@ __global__ void __launch_bounds__(kTlThreads, 1) tiles_kernel(const __grid_const
     const float *c1 = S + (size_t)b * R * W, *c0 = S + (size_t)(b ^ 1) * R * W;
     bool bad = false;
     if constexpr (!TRAJ) {
-        // ---- the end: C^{n+k} and C^{n+k-1} go out.  One of them overwrites the input: after an
-        // exchange every neighbour is known to have loaded its tile, else its flag says so
+        // ---- the end: C^{n+k} and C^{n+k-1} go out.  One of them overwrites the input: every
+        // neighbour's flag says that it has loaded its tile (looked at in the first exchange, or here)
         if (nrounds == 1 && warp == 0) {
             const bool ok = wait_neighbours(A, T.tx, T.ty, A.base);
             if (lane == 0) s_push = ok ? 0 : -1;

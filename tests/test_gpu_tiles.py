@@ -178,6 +178,31 @@ def test_stored_states_of_tiles_that_are_crowded_now_and_then(cue, depth, rate_m
         assert np.array_equal(plain[k], tiles[k]), k
 
 
+@pytest.mark.parametrize("name,depth,chunk", [
+    ("512x300-clamp-4000cones", 0, 1), ("515x301-stop-4000cones", 0, 1), ("515x301-stop-4000cones", 1, 2),
+    ("640x400-crowd-stop-5000cones", 0, 1), ("644x400-crowd-clamp-5000cones", 0, 3),
+])
+def test_many_short_runs_find_every_cone_once(cue, name, depth, chunk):
+    """The cones are found anew by every run, from arrays that the run's other blocks are about to write. Cones cross
+    tile borders all the time; the caches are cold before each run, so that blocks load at different speeds."""
+    import torch
+    w = _case(name)
+    w.w_grad, w.w_noise = 0.1, 0.5
+    flush = torch.empty(96 << 20, dtype=torch.int32, device="cuda:0")
+    a = cue.Simulation(w, path=cue.CUE_PATH_PLAIN)
+    b = cue.Simulation(w, path=cue.CUE_PATH_AUTO if w.nx % 4 else cue.CUE_PATH_PERSIST)
+    b.set_option(cue.CUE_OPT_TEMPORAL_DEPTH, depth)
+    for k in range(60):
+        a.sim_run(chunk)
+        flush.fill_(k)
+        b.sim_run(chunk)
+        b.check()
+        _assert_same(a.snapshot(), b.snapshot())
+    assert b.get_option(cue.CUE_INFO_GRID) > 1 and a.cone_updates() == b.cone_updates()
+    a.close()
+    b.close()
+
+
 def test_device_side_problems_are_reported(cue):
     """Non-finite input is reported; sources outside the grid are skipped and reported."""
     w = _case("512x300")
