@@ -33,7 +33,10 @@
 // global memory, and all warps share them out by a ticket.  At the end of a round
 // a cone that left the interior is posted to the neighbour it went to: the first
 // kTlPost per neighbour with their state, more through the tile's inbox (ids;
-// state through the caller's arrays).
+// state through the caller's arrays).  An inbox is ordinary memory: who put
+// cones into one fences before the number that tells of it, and a tile that took cones from its
+// own fences before its next number and says so in it (kTlInboxUsed), on which the neighbours
+// fence before they may add to that inbox again.
 //
 // All tiles have one shape, W = 128 columns (one float4 per lane) by R rows, always inside the
 // grid (the last tile of an axis is shifted inwards), so a wall is always the
@@ -86,6 +89,7 @@ constexpr int kTlMaxSrc = 1024;
 constexpr int kTlW = 128;                    // loaded columns: one float4 per lane
 constexpr int kTlMaxRows = 15;               // rows of a field warp, in registers
 constexpr int kTlPost = kTilesPost;          // cones posted with their state per neighbour and round
+constexpr unsigned kTlInboxUsed = 1u << 31;  // beside the number of posted cones
 constexpr int kTlCrowdMin = 512;             // runs of fewer cones are never too crowded
 constexpr int kTlFlagWords = 64;             // a flag's stride: a line of its own
 constexpr int kTlInFlight = 4;               // rows whose packets a warp polls together
@@ -806,8 +810,9 @@ __device__ __forceinline__ unsigned cone_loop(const TileArgs &A, const Tile &T, 
             asm volatile("bar.sync 1, %0;" ::"r"(kTlOwn) : "memory");      // the cone warps have placed theirs
             if (cw == 0 && lane < 9) {
                 const int c = s_out[lane];
-                if (c > kTlPost) __threadfence();
-                if (nb) st_packet(post_box(A, par, ny * A.gx + nx, 8 - lane) + 3 * kTlPost, packet((unsigned)c, tag));
+                const bool used = ovf0 + n_ovf > 0;     // this round's list came from the inbox, in part
+                if (c > kTlPost || used) __threadfence();
+                if (nb) st_packet(post_box(A, par, ny * A.gx + nx, 8 - lane) + 3 * kTlPost, packet((unsigned)c | (used ? kTlInboxUsed : 0u), tag));
                 s_out[lane] = 0;
             }
         }
@@ -826,7 +831,8 @@ __device__ __forceinline__ unsigned cone_loop(const TileArgs &A, const Tile &T, 
                         ok = keep_waiting(it, A.limit, A.abort, A.base, A.status);
                         w = ld_packet(q);
                     }
-                    c = ok ? (int)(unsigned)w : 0;
+                    c = ok ? (int)((unsigned)w & ~kTlInboxUsed) : 0;
+                    if ((unsigned)w & kTlInboxUsed) __threadfence();
                 }
                 // cones in the inbox: from a neighbour that had more than it can post, or this tile's own
                 const int stayed = *s_push;
@@ -835,9 +841,8 @@ __device__ __forceinline__ unsigned cone_loop(const TileArgs &A, const Tile &T, 
                 int in_box = 0;
                 if (__any_sync(kFull, c > kTlPost) || stayed > cap) {
                     __threadfence();
-                    in_box = min(__ldcg(A.cnt_cur + np * kTilesMax + T.t), n);
-                    __syncwarp();
-                    if (lane == 0) A.cnt_cur[np * kTilesMax + T.t] = 0;
+                    if (lane == 0) in_box = min(atomicExch(A.cnt_cur + np * kTilesMax + T.t, 0), n);
+                    in_box = __shfl_sync(kFull, in_box, 0);
                 }
                 c = min(c, kTlPost);
                 int upto = c;                           // posted cones from neighbours up to this lane's

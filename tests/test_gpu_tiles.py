@@ -181,6 +181,7 @@ def test_stored_states_of_tiles_that_are_crowded_now_and_then(cue, depth, rate_m
 @pytest.mark.parametrize("name,depth,chunk", [
     ("512x300-clamp-4000cones", 0, 1), ("515x301-stop-4000cones", 0, 1), ("515x301-stop-4000cones", 1, 2),
     ("640x400-crowd-stop-5000cones", 0, 1), ("644x400-crowd-clamp-5000cones", 0, 3),
+    ("640x400-crowd-clamp-5000cones", 1, 2), ("640x401-crowd-stop-5000cones", 4, 7),
 ])
 def test_many_short_runs_find_every_cone_once(cue, name, depth, chunk):
     """The cones are found anew by every run, from arrays that the run's other blocks are about to write. Cones cross
@@ -201,6 +202,20 @@ def test_many_short_runs_find_every_cone_once(cue, name, depth, chunk):
     assert b.get_option(cue.CUE_INFO_GRID) > 1 and a.cone_updates() == b.cone_updates()
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("depth", [1, 2, 6])
+@pytest.mark.parametrize("name", ["640x400-crowd-clamp-8000cones", "640x400-crowd-stop-3000cones"])
+def test_a_crowd_that_marches_through_tiles(cue, name, depth):
+    """All cones go the same way, from tile to tile: far more than a neighbour is posted, in lists that are longer than
+    shared memory holds, so that every inbox on the way is filled, emptied and filled again."""
+    w = _case(name)
+    w.w_prev, w.w_grad, w.w_noise = 1.0, 0.0, 0.02
+    w.dir[0], w.dir[1] = 0.6, -0.8
+    a, _ = _run(cue, w, cue.CUE_PATH_PLAIN, [130])
+    b, (path, _) = _run(cue, w, cue.CUE_PATH_PERSIST, [90, 40], depth=depth)
+    assert path == cue.CUE_PATH_PERSIST
+    _assert_same(a, b)
 
 
 def test_device_side_problems_are_reported(cue):
