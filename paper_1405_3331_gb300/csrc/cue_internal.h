@@ -2,6 +2,7 @@
 // libcue.so (handle layout, workspace layout, kernel launchers).
 #pragma once
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <cuda.h>
@@ -45,6 +46,32 @@ struct WorkspaceLayout {
     size_t total = 0;
     int n_tiles = 0;
     int bin_cap = 0;             // cone ids per tile bin
+};
+
+// A number (>= 0) that is found once per device: what a kernel was allowed and how much of it fits belong to the device
+// that was current.  Safe with several threads (they may find it twice, and find the same).
+class PerDevice {
+public:
+    template <class F> int on(int dev, const F &find)
+    {
+        if (dev < 0 || dev >= kDevices) return find();
+        int v = known_[dev].load(std::memory_order_acquire);
+        if (v == 0) {
+            v = find() + 1;
+            known_[dev].store(v, std::memory_order_release);
+        }
+        return v - 1;
+    }
+    template <class F> int on_current(const F &find)
+    {
+        int dev = -1;
+        if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+        return on(dev, find);
+    }
+
+private:
+    static constexpr int kDevices = 64;
+    std::atomic<int> known_[kDevices] = {};              // the number + 1; 0: not found yet
 };
 
 // ---- the persistent path's tile engine (k_tiles.cu) ----

@@ -600,10 +600,8 @@ __global__ void __launch_bounds__(kBfsThreads) bfs_cluster_kernel(int nv, const 
 int bfs_smem(int nv, int G) { return (2 * kBfsQueue + (nv / G + 32) / 32 + 1) * (int)sizeof(int); }
 
 // Blocks of the cluster the search starts on: 16 where the device can schedule it, else 8, else 0 (none).
-int bfs_cluster_size()
+int bfs_find_cluster_size()
 {
-    static int size = -1;
-    if (size >= 0) return size;
     const int smem = bfs_smem(kBfsMaxVertices, 16);
     int best = 0;
     if (cudaFuncSetAttribute(bfs_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
@@ -622,9 +620,14 @@ int bfs_cluster_size()
             int n = 0;
             if (cudaOccupancyMaxActiveClusters(&n, bfs_cluster_kernel, &cfg) == cudaSuccess && n > 0) best = g;
         }
-    cudaGetLastError();                                  // a size the device refuses is no error of the caller's
-    size = best;
-    return size;
+    if (best < 16) cudaGetLastError();                   // a size the device refuses is no error of the caller's
+    return best;
+}
+
+int bfs_cluster_size()
+{
+    static PerDevice size;
+    return size.on_current(bfs_find_cluster_size);
 }
 
 cudaError_t launch_bfs_cluster(int G, int nv, const int *row, const int *col, int source, int *level, int *state, cudaStream_t st)

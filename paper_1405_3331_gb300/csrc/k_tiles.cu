@@ -1134,14 +1134,13 @@ __global__ void __launch_bounds__(kTlThreads, 1) tiles_kernel(const __grid_const
 
 int sm_count_t()
 {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
+    static PerDevice count;
+    return count.on_current([] {
+        int dev = 0, n = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 152;
-    }
-    return n;
+        return n > 0 ? n : 152;
+    });
 }
 
 constexpr size_t kTlSmemMax = 227u * 1024u - 3072u;     // a block's limit, less the kernel's static shared memory
@@ -1220,16 +1219,30 @@ bool tiles_geometry(const FieldDesc &f, float step_len, bool map, bool vec, int 
 static size_t tiles_flags_bytes() { return (sizeof(unsigned) * ((kTlFlagWords + 4) * kTilesMax + 64) + 255) & ~(size_t)255; }
 size_t tiles_ctl_bytes() { return tiles_flags_bytes() + sizeof(ulonglong2) * 2 * kTilesMax * 9 * (3 * kTlPost + 1); }
 
+// The kernel's shared-memory allowance on the current device; false where it is refused (the grid then takes the
+// path that the engine would have displaced).
+template <bool MAP, bool TRAJ, bool VEC>
+static bool tiles_allowed_t()
+{
+    static PerDevice allowed;
+    return allowed.on_current([] {
+        if (cudaFuncSetAttribute(tiles_kernel<MAP, TRAJ, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTlSmemMax) == cudaSuccess)
+            return 1;
+        cudaGetLastError();
+        return 0;
+    }) == 1;
+}
+
+template <bool TRAJ>
+static bool tiles_allowed(const Sim &s)
+{
+    if (s.vec4) return s.src_map ? tiles_allowed_t<true, TRAJ, true>() : tiles_allowed_t<false, TRAJ, true>();
+    return s.src_map ? tiles_allowed_t<true, TRAJ, false>() : tiles_allowed_t<false, TRAJ, false>();
+}
+
 template <bool MAP, bool TRAJ, bool VEC>
 static cudaError_t tiles_launch_t(const TileArgs &A, int grid, size_t smem, cudaStream_t stream)
 {
-    static bool ready = false;
-    if (!ready) {
-        cudaError_t e = cudaFuncSetAttribute(tiles_kernel<MAP, TRAJ, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kTlSmemMax);
-        if (e != cudaSuccess) return e;
-        ready = true;
-    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kTlThreads);
@@ -1243,6 +1256,7 @@ static cudaError_t tiles_launch_t(const TileArgs &A, int grid, size_t smem, cuda
     return cudaLaunchKernelEx(&cfg, tiles_kernel<MAP, TRAJ, VEC>, A);
 }
 
+template <bool TRAJ = false>
 static bool tiles_ready(Sim &s, TilesGeom &g)
 {
     // the work-list kernel's own options, its phantom arrivals and stream captures stay with it
@@ -1253,7 +1267,7 @@ static bool tiles_ready(Sim &s, TilesGeom &g)
         s.tiles_geom_ready = true;
         s.tiles_geom_depth = s.temporal_depth;
     }
-    if (!s.tiles_geom_ok) return false;
+    if (!s.tiles_geom_ok || !tiles_allowed<TRAJ>(s)) return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
     g = s.tiles_geom;
@@ -1390,7 +1404,7 @@ int run_tiles_if_supported(Sim &s, int nsteps)
 int run_tiles_trajectory(Sim &s, float *traj_field, float *traj_cone, uint32_t step0, int nsteps)
 {
     TilesGeom g;
-    if (!tiles_ready(s, g) || nsteps > kPersistMaxSteps) return 1;
+    if (!tiles_ready<true>(s, g) || nsteps > kPersistMaxSteps) return 1;
     return tiles_launch(s, g, nsteps, step0, traj_field, traj_cone);
 }
 
