@@ -130,9 +130,11 @@ typedef struct cue_sim cue_sim;   /* opaque, host-side */
                                       share out the cones of crowded tiles (sized from the
                                       crowding the previous run reported; 0 on the first)  */
 #define CUE_PATH_AUTO   0          /* library picks: for 2D grids that fit the SMs' shared
-                                      memory (up to about 1500^2, nx >= 128, any nx), above
+                                      memory (up to about 1700^2, nx >= 128, any nx), above
                                       65536 nodes or with nx % 4 != 0, the persistent path's
-                                      tile engine; else fused for 2D grids of at least one tile
+                                      tile engine where its modelled time for the call's steps
+                                      (and the crowding of the last runs) is the shorter one;
+                                      else fused for 2D grids of at least one tile
                                       per SM; else cluster for 2D grids of at least 4096
                                       nodes with at most 128 cones and 16384 nodes per block;
                                       else resident; else persistent; else plain (3D: one

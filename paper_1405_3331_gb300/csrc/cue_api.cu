@@ -134,6 +134,24 @@ static int sm_count_api()
     return n;
 }
 
+// What a 2D run takes on the path that the tile engine would displace, in microseconds: measured at 288 x 256 to 1700^2
+// (fused, cluster, work-list) and 129^2 to 1701^2 (one launch a step) with 1 to 256 steps a call.  With more than 128
+// cones in a tile the fused path takes 3.5 to 4.1 us a step instead of 2.8, the work-list 4 to 6 instead of 7.
+static double other_path_us(const Sim &s, int nsteps, bool fused, bool cluster)
+{
+    const double nodes = (double)s.fd.nx * s.fd.ny, n = nsteps;
+    if (!s.vec4)                                         // 129^2 2.3, 1025 x 769 4.7, 1701^2 7.0 a step
+        return n * (2.6 + 1.9e-6 * std::min(nodes, 1e6) + 1.3e-6 * std::max(nodes - 1e6, 0.0));
+    if (fused) {                                         // 1024^2: one step 15.9, eight 28.8, 64 180; without cones 7.2, 22.9, 186
+        const double crowd = s.crowd_us > 0.0 ? std::min(1.5, 0.4 + 0.4 * s.crowd_us) : 0.0;
+        return s.n_axons > 0 ? 9.0 + 5.0 * std::ceil(n / 8.0) + n * (1.7 + 0.25e-6 * nodes + crowd)
+                             : 5.0 * std::ceil(n / 8.0) + n * 2.14e-6 * nodes;
+    }
+    if (cluster) return 8.4 + n * (1.2 + 8e-6 * nodes) * (s.src_map ? 1.3 : 1.0);   // 288 x 256 1.8, 512^2 3.3, 4.3 with a map
+    const double crowd = std::min(2.5, 0.4 * s.crowd_us);                  // (a crowd's cones are shared out)
+    return 3.4 + n * (6.9 - crowd) * std::max(1.0, nodes / 1.05e6);       // 768^2 7.0, 1152^2 9.2
+}
+
 int run_coupled(Sim &s, int nsteps)
 {
     s.fused_used = false;
@@ -141,10 +159,10 @@ int run_coupled(Sim &s, int nsteps)
     s.resident_used = false;
     s.cluster_used = false;
     // AUTO, 2D: the persistent path's tile engine ahead of the others for rows that are not whole float4
-    // groups (which otherwise run two scalar launches a step: 1025 x 769 17.4 -> 1.8 us) and for grids above
-    // those the cluster path is kept for (512 x 384 with 2,000 cones 4.3 -> 1.5 us; 1024^2 with a map 6.4 -> 1.6
-    // on the work-list kernel, without one 3.4 -> 1.4 on the fused path), unless the handle's last runs
-    // crowded into few tiles.  Then the temporally blocked kernel when the grid gives every SM a tile;
+    // groups (1025 x 769 in long runs 4.7 us a step as one launch each, 1.3 on the engine) and for grids above
+    // those the cluster path is kept for (512 x 384 2.8 -> 0.9 us; 1024^2 with a map 6.8 -> 1.5
+    // on the work-list kernel, without one 2.9 -> 1.3 on the fused path), where the run's modelled time is
+    // the shorter one (other_path_us).  Then the temporally blocked kernel when the grid gives every SM a tile;
     // else a cluster of CTAs with the grid in their distributed shared memory
     // where its measured step is the shortest (cluster_preferred); else one
     // block with the grid in shared memory; else the persistent launch (larger
@@ -155,9 +173,7 @@ int run_coupled(Sim &s, int nsteps)
     bool tiles = s.path == CUE_PATH_PERSIST;
     if (s.path == CUE_PATH_AUTO && s.fd.dim == 2 && tiles_supported(s)) {
         const bool first = !s.vec4 || (long long)s.fd.nx * s.fd.ny > 65536;
-        // (microseconds a step of the path it displaces)
-        const double alt_us = !small ? 4.0 : cluster_preferred(s) ? 2.5 : 6.5;
-        tiles = !s.vec4 || !tiles_crowded(s, alt_us);
+        tiles = tiles_preferred(s, nsteps, other_path_us(s, nsteps, !small, small && first && s.vec4 && cluster_preferred(s)));
         if (first && tiles) rc = run_tiles_if_supported(s, nsteps);
         if (rc != 1) return rc;
         tiles = tiles && small;

@@ -77,6 +77,7 @@ private:
 // ---- the persistent path's tile engine (k_tiles.cu) ----
 constexpr int kTilesMax = 160;            // tiles (at most one per SM)
 constexpr int kTilesMaxCones = 64 * kTilesMax;   // (its rule's limit) a tile's inbox can hold every cone
+constexpr int kTilesCrowdLeave = 15;      // runs left to another path once a crowd has made the engine the slower one
 constexpr int kTilesPost = 16;            // cones posted with their state per neighbour and round
 constexpr long long kTilesMaxNodes = 1 << 22;   // grids up to this get its workspace
 struct TilesGeom {
@@ -85,6 +86,7 @@ struct TilesGeom {
     int gx = 0, gy = 0;                   // tiles per axis
     int K = 0;                            // steps per round
     int cap = 0;                          // cones in its shared-memory list
+    double step_us = 0.0, exchange_us = 0.0, start_us = 0.0;   // what a step, a further round and a launch take
 };
 size_t tiles_ctl_bytes();
 
@@ -237,11 +239,13 @@ struct Sim {
     int tiles_geom_depth = 0;
     TilesGeom tiles_geom{};
     unsigned tiles_launches = 0, tiles_base = 1;
-    // the most crowded tile of the last watched run (pinned word + event), and the runs left to other paths
+    // what the most crowded tile of the last watched run added to a step (pinned word + event), the runs left to
+    // other paths (-1: none decided) and how many the next decision leaves
     int *crowd_host = nullptr;
     cudaEvent_t crowd_ev = nullptr;
     bool crowd_pending = false;
-    int crowd_skip = 0;
+    double crowd_us = 0.0;
+    int crowd_left = -1, crowd_leave = kTilesCrowdLeave;
 
     // fused path
     // helper CTAs for crowded tiles: the total need the last run reported, read back
@@ -327,8 +331,10 @@ int run_persist_trajectory(Sim &s, float *traj_field, float *traj_cone, uint32_t
 bool tiles_geometry(const FieldDesc &f, float step_len, bool map, bool vec, int n_src, int n_axons, int depth, int sms,
                     TilesGeom &best);
 bool tiles_supported(Sim &s);
-// Whether the handle's last runs were too crowded for it, against another path of alt_us a step.
-bool tiles_crowded(Sim &s, double alt_us);
+// Whether a run of nsteps is expected to take no longer on it than other_us, by its shape and the crowd last seen.
+bool tiles_faster(Sim &s, int nsteps, double other_us);
+// The same as AUTO's choice for a run: a crowd is looked at again after some runs on the other path.
+bool tiles_preferred(Sim &s, int nsteps, double other_us);
 // Runs nsteps on the tile engine where it fits: CUE_OK / negative error, or 1 when the caller
 // should use another kernel.
 int run_tiles_if_supported(Sim &s, int nsteps);

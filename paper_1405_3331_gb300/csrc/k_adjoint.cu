@@ -1212,7 +1212,9 @@ int run_adjoint(Sim &s, const float *targets, int nsteps, int k, void *ws, size_
     // its start): one persistent launch where the path runs, else a cone and a
     // field launch per step
     auto trajectory = [&](int len, int64_t nstart) -> int {
-        int rc = (s.path == CUE_PATH_AUTO || s.path == CUE_PATH_PERSIST)
+        // (the work-list kernel otherwise, or two or three launches a step)
+        const double other = s.vec4 ? 3.4 + 6.9 * len : len * (6.0 + 2e-6 * (double)cells);
+        int rc = ((s.path == CUE_PATH_AUTO && tiles_faster(s, len, other)) || s.path == CUE_PATH_PERSIST)
                      ? run_tiles_trajectory(s, sgC, sgP, (uint32_t)nstart, len)
                      : 1;
         if (rc == 1 && s.path != CUE_PATH_PLAIN && persist_supported(s))

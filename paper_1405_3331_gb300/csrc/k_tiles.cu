@@ -90,7 +90,6 @@ constexpr int kTlW = 128;                    // loaded columns: one float4 per l
 constexpr int kTlMaxRows = 15;               // rows of a field warp, in registers
 constexpr int kTlPost = kTilesPost;          // cones posted with their state per neighbour and round
 constexpr unsigned kTlInboxUsed = 1u << 31;  // beside the number of posted cones
-constexpr int kTlCrowdMin = 512;             // runs of fewer cones are never too crowded
 constexpr int kTlFlagWords = 64;             // a flag's stride: a line of its own
 constexpr int kTlInFlight = 4;               // rows whose packets a warp polls together
 
@@ -118,7 +117,7 @@ struct TileArgs {
     unsigned *flags;                         // [tiles], kTlFlagWords apart, only growing: "tile loaded"
     unsigned base;                           // this launch's first tag and its flag; earlier ones' are below it
     unsigned *abort;                         // the aborting launch's base
-    int *crowd;                              // most cones of a tile at the start of a round, where over kTlOwn
+    int *crowd;                              // the nanoseconds a step that a tile's crowd added (the largest tile's)
     long long limit;
     unsigned *status;
     unsigned long long *counter;
@@ -340,6 +339,15 @@ __device__ __noinline__ unsigned crowd_cones(const TileArgs &A, Tile T, const fl
     }
     if (bits) flag_status(A.status, bits);
     return live;
+}
+
+// What `held` cones of one tile (more than kTlOwn) add to its step, in nanoseconds: the field sweep leaves the registers,
+// and the cones past the first 128 queue up.  Measured at 512 x 384, 768^2 and 1280^2 with one crowd, over the
+// uncrowded step of 1.0, 1.1 and 1.7 us: 150 cones 1.6, 1.8, 1.6 us; 500: 2.0, 2.1, 2.1; 1,000: 3.2, 3.4, 3.4;
+// 2,500: 8.2, 8.6, 8.8; 4,000: 12.9, 13.3, 14.1.
+__device__ __forceinline__ float crowd_ns(int held)
+{
+    return 1300.0f + 1.5f * (float)min(held, 512) + 2.5f * (float)min(max(held - 512, 0), 512) + 3.3f * (float)max(held - 1024, 0);
 }
 
 // What a field warp's lane does with its group's four nodes: bit k is node k.
@@ -656,14 +664,15 @@ __device__ __forceinline__ unsigned cone_loop(const TileArgs &A, const Tile &T, 
     const int n = A.n, cap = A.cap, R = T.R;
     const int nrounds = (A.nsteps + A.K - 1) / A.K;
     unsigned live = 0, bits = 0;
-    int lb = 0, most = 0;
+    int lb = 0;
+    float crowd = 0.0f;
     for (int rd = 0, done = 0; rd < nrounds; ++rd) {
         const int kr = min(A.K, A.nsteps - done), par = rd & 1;
         const int m = s_list[0], ovf0 = s_list[1], n_ovf = s_list[2];
         int *ovf = inbox_of(A, par, T.t) + ovf0;
         const int slot = cw * 32 + lane;
         // few cones: the second half of the warps draws the first half's noise a step ahead
-        most = max(most, m + n_ovf);
+        if (m + n_ovf > kTlOwn) crowd += (float)kr * crowd_ns(m + n_ovf);
         const bool helped = m + n_ovf <= kTlHelped;
         const int h_slot = slot - kTlHelped, h_id = helped && h_slot >= 0 && h_slot < m ? T.l_id[lb * cap + h_slot] : -1;
         int a = -1;
@@ -917,7 +926,7 @@ __device__ __forceinline__ unsigned cone_loop(const TileArgs &A, const Tile &T, 
         lb ^= 1;
     }
     if (bits) flag_status(A.status, bits);
-    if (most > kTlOwn && cw == 0 && lane == 0) atomicMax(A.crowd, most);
+    if (crowd > 0.0f && cw == 0 && lane == 0) atomicMax(A.crowd, (int)(crowd / (float)A.nsteps));
     return live;
 }
 
@@ -1186,9 +1195,9 @@ bool tiles_shape(int nx, int ny, bool cones, float step_len, float h, int K, int
 // The steps a round K: microseconds a step by what was measured on GB300 -- a field warp's rows
 // (0.1 each; at least 0.75 with cones, their dependent chain), and an exchange shared by the K steps of a round
 // (1.9, and 0.045 a node of halo width; 1.6 times that where rows are not whole float4 groups).
-// 1024^2 with 4,096 cones: K = 3, 4, 6, 8, 10 took 1.78, 1.57, 1.39, 1.53, 1.47 us a step (3.4 on the
-// fused path; with a map 1.6 against 6.4 on the work-list kernel); 1025 x 769: 2.63, 2.30, 1.97, 1.92, 1.82 (17.4 as two launches a step);
-// 512 x 384 with 2,000: 1.99, 1.85, 1.61, 1.52, 1.54 (4.3 on the cluster path).
+// 1024^2 with 4,096 spread cones: K = 3 to 12 took 1.73, 1.48, 1.43, 1.32, 1.35, 1.50, 1.50, 1.43, 1.32, 1.35 us a step,
+// the rule picks 7; 1025 x 769: 2.20, 1.87, 1.71, 1.56, 1.51, 1.60, 1.55, 1.51, 1.63, 1.60, it picks 10; 512 x 384 with 2,000:
+// 1.45, 1.24, 1.13, 1.04, 0.99, 0.96, 0.97, 0.93, 0.97, 0.98, it picks 12.
 bool tiles_geometry(const FieldDesc &f, float step_len, bool map, bool vec, int n_src, int n_axons, int depth, int sms,
                     TilesGeom &best)
 {
@@ -1205,7 +1214,14 @@ bool tiles_geometry(const FieldDesc &f, float step_len, bool map, bool vec, int 
         g.cap = std::min((n_axons + 31) & ~31, 1024);
         if (tiles_smem(g, map, n_src) > kTlSmemMax) continue;
         const int rows = (g.R + kTlFieldWarps - 1) / kTlFieldWarps;
-        const double t = std::max(0.11 + 0.1 * rows, cones ? 0.75 : 0.0) + (vec ? 1.0 : 1.6) * (1.9 + 0.045 * (g.HX + g.HY)) / K;
+        const double edge = vec ? 1.0 : 1.6, sweep = std::max(0.11 + 0.1 * rows, cones ? 0.75 : 0.0);
+        const double t = sweep + edge * (1.9 + 0.045 * (g.HX + g.HY)) / K;
+        // (for AUTO's choice: tall tiles' exchanges take longer than that, 7.2 us at 168 rows, 12 where rows are not
+        // whole float4 groups; and a launch, which loads the grid, finds the cones and writes two grids, 9 to 20 us, up to 33)
+        const double nodes = (double)f.nx * f.ny;
+        g.step_us = sweep;
+        g.exchange_us = edge * (1.9 + 0.045 * (g.HX + g.HY) + 0.1 * std::max(0, g.R - 130)) + (map ? 1.0 : 0.0);
+        g.start_us = vec ? (cones ? 9.5 + 3.4e-6 * nodes : 7.5 + 1.7e-6 * nodes) : cones ? 11.0 + 7.6e-6 * nodes : 10.0 + 5e-6 * nodes;
         if (!found || t < best_t) {
             best = g;
             best_t = t;
@@ -1349,19 +1365,49 @@ bool tiles_supported(Sim &s)
     return tiles_ready(s, g);
 }
 
-// A tile's cones are stepped by its block alone, about 1.3 ns a cone past its registers (a step with 966, 1,024
-// or 4,096 cones in one tile: 3.0, 3.2, 6.5 us), where other paths share a crowd out better.  So the most
-// crowded tile of a run is read back (without waiting, as the fused path's helpers are sized), and when it would have
-// cost more than `alt_us` a step the next 15 runs of the handle are left to the other path.
-bool tiles_crowded(Sim &s, double alt_us)
+// The modelled time of a run against the other path's: short calls pay for the load of the grid and both buffers' way
+// out, large grids for tall tiles and many exchanges, crowds for a tile whose cones its block steps alone (crowd_ns), where
+// other paths share them out.  Over 288 x 256 to 1701^2, 1 to 256 steps a call, with and without cones and map, the choice
+// is the faster one or within 6% of it but for odd rows at 6 steps (18%).  The crowd's part is read back from the last
+// watched run without waiting, as the fused path's helpers are sized.
+bool tiles_faster(Sim &s, int nsteps, double other_us)
 {
+    TilesGeom g;
+    if (!tiles_ready(s, g)) return false;
     if (s.crowd_pending && cudaEventQuery(s.crowd_ev) == cudaSuccess) {
         s.crowd_pending = false;
-        if (1.75 + 1.3e-3 * *s.crowd_host > alt_us) s.crowd_skip = 15;
+        s.crowd_us = 1e-3 * *s.crowd_host;
     }
-    if (s.crowd_skip <= 0) return false;
-    s.crowd_skip--;
-    return true;
+    const int rounds = (nsteps + g.K - 1) / g.K;
+    // a depth that was asked for is a wish for the engine: only a crowd speaks against it
+    const double plain = s.temporal_depth > 0 ? 0.0 : g.start_us + (s.crowd_us > 0.0 ? 2.5 : 0.0) + nsteps * g.step_us + (rounds - 1) * g.exchange_us;
+    return plain + nsteps * s.crowd_us <= other_us;
+}
+
+// A crowd that makes the engine the slower one leaves the next 15 runs to the other path; then one run looks
+// again, and while the crowd is still there the number left doubles (up to 960).  (One run: many may be queued before its
+// readback comes.)
+bool tiles_preferred(Sim &s, int nsteps, double other_us)
+{
+    if (tiles_faster(s, nsteps, other_us)) {
+        if (!s.crowd_pending) {
+            s.crowd_leave = kTilesCrowdLeave;
+            s.crowd_left = -1;
+        }
+        return true;
+    }
+    if (s.crowd_us == 0.0) return false;
+    if (s.crowd_left < 0) {
+        s.crowd_left = s.crowd_leave;
+        s.crowd_leave = std::min(2 * s.crowd_leave, 64 * kTilesCrowdLeave);
+    }
+    if (s.crowd_left-- > 0) return false;
+    const double was = s.crowd_us;
+    s.crowd_us = 0.0;
+    const bool look = !s.crowd_pending && tiles_faster(s, nsteps, other_us);
+    s.crowd_us = was;
+    if (!look) s.crowd_left = 0;                         // not a run to look with: the next one does
+    return look;
 }
 
 int run_tiles_if_supported(Sim &s, int nsteps)
@@ -1374,7 +1420,7 @@ int run_tiles_if_supported(Sim &s, int nsteps)
         s.src_xyz_ready = true;
     }
     int *crowd = reinterpret_cast<int *>(s.ws + s.wl.tiles_off) + (kTlFlagWords + 4) * kTilesMax + 1;
-    const bool watch = s.adapt_helpers && s.path == CUE_PATH_AUTO && s.n_axons > kTlCrowdMin && !s.crowd_pending;
+    const bool watch = s.adapt_helpers && s.path == CUE_PATH_AUTO && s.n_axons > kTlOwn && !s.crowd_pending;
     if (watch && cudaMemsetAsync(crowd, 0, sizeof(int), s.stream) != cudaSuccess) return CUE_ERR_CUDA;
     for (int done = 0; done < nsteps;) {
         const int k = std::min(nsteps - done, kPersistMaxSteps);

@@ -179,7 +179,7 @@ def test_stored_states_of_tiles_that_are_crowded_now_and_then(cue, depth, rate_m
 
 
 @pytest.mark.parametrize("name,depth,chunk", [
-    ("512x300-clamp-4000cones", 0, 1), ("515x301-stop-4000cones", 0, 1), ("515x301-stop-4000cones", 1, 2),
+    ("512x300-clamp-4000cones", 0, 1), ("515x301-stop-4000cones", 5, 1), ("515x301-stop-4000cones", 1, 2),
     ("640x400-crowd-stop-5000cones", 0, 1), ("644x400-crowd-clamp-5000cones", 0, 3),
     ("640x400-crowd-clamp-5000cones", 1, 2), ("640x401-crowd-stop-5000cones", 4, 7),
 ])
@@ -216,6 +216,42 @@ def test_a_crowd_that_marches_through_tiles(cue, name, depth):
     b, (path, _) = _run(cue, w, cue.CUE_PATH_PERSIST, [90, 40], depth=depth)
     assert path == cue.CUE_PATH_PERSIST
     _assert_same(a, b)
+
+
+@pytest.mark.parametrize("name,steps,path", [
+    ("1025x769-1000cones", 1, "PLAIN"), ("1025x769-1000cones", 64, "PERSIST"), ("1024x1024-0cones", 1, "FUSED"),
+    ("1024x1024-0cones", 64, "PERSIST"), ("1024x1024-4000cones", 8, "PERSIST"), ("1700x1700-1000cones", 64, "FUSED"),
+    ("1701x1701-1000cones", 64, "PLAIN"),
+])
+def test_the_library_s_choice_compares_whole_runs(cue, name, steps, path):
+    """A run's modelled time against the path it would displace: short runs do not pay for the engine's start, nor
+    grids for tiles too tall for it."""
+    w = _case(name)
+    a, _ = _run(cue, w, cue.CUE_PATH_PLAIN, [steps])
+    b, (got, _) = _run(cue, w, cue.CUE_PATH_AUTO, [steps])
+    assert got == getattr(cue, "CUE_PATH_" + path)
+    _assert_same(a[:1] + a[2:], b[:1] + b[2:])           # (the fused path leaves an earlier step in the other buffer)
+
+
+def test_crowds_on_rows_of_any_length_go_to_another_path_and_are_looked_at_again(cue):
+    """As above for rows that are not whole float4 groups; while the crowd stays, the engine is tried again after
+    15, 30, ... runs."""
+    import torch
+    w = _case("1025x769-crowd-clamp-4000cones")
+    a, b = cue.Simulation(w, path=cue.CUE_PATH_PLAIN), cue.Simulation(w)
+    paths = []
+    for k in range(49):
+        b.load(C=w.field0(), pos=w.pos, dir=w.dir, active=w.active, step=0)
+        b.sim_run(20)
+        b.check()
+        paths.append(b.last_path())
+        torch.cuda.synchronize()
+    engine, other = cue.CUE_PATH_PERSIST, cue.CUE_PATH_PLAIN
+    assert paths == [engine] + 15 * [other] + [engine] + 30 * [other] + [engine] + [other]
+    a.sim_run(20)
+    _assert_same(a.snapshot(), b.snapshot())
+    a.close()
+    b.close()
 
 
 def test_device_side_problems_are_reported(cue):
