@@ -49,8 +49,8 @@ WorkspaceLayout workspace_layout(const cue_params &p, int n_src, int n_axons)
         off += align256(sizeof(float) * (size_t)p.nx * p.ny * p.nz);
     }
     w.base_total = off;
-    // the tile engine's flags and inboxes, for the 2D grids it can hold
-    if (p.dim == 2 && p.nx >= 128 && (long long)p.nx * p.ny <= kTilesMaxNodes && n_axons <= kTilesMaxCones) {
+    // the tile engine's flags and inboxes, for the 2D grids it can hold (2048^2, which it cannot, does without 67 MB)
+    if (p.dim == 2 && n_axons <= kTilesMaxCones && tiles_possible(p.nx, p.ny, n_axons > 0)) {
         w.tiles_off = off;
         off += align256(tiles_ctl_bytes());
         w.tiles_packets_off = off;

@@ -79,7 +79,6 @@ constexpr int kTilesMax = 160;            // tiles (at most one per SM)
 constexpr int kTilesMaxCones = 64 * kTilesMax;   // (its rule's limit) a tile's inbox can hold every cone
 constexpr int kTilesCrowdLeave = 15;      // runs left to another path once a crowd has made the engine the slower one
 constexpr int kTilesPost = 16;            // cones posted with their state per neighbour and round
-constexpr long long kTilesMaxNodes = 1 << 22;   // grids up to this get its workspace
 struct TilesGeom {
     int W = 0, R = 0;                     // loaded columns (128 s), rows
     int HX = 0, HY = 0;                   // halo
@@ -89,6 +88,8 @@ struct TilesGeom {
     double step_us = 0.0, exchange_us = 0.0, start_us = 0.0;   // what a step, a further round and a launch take
 };
 size_t tiles_ctl_bytes();
+// Whether any tiling of the grid fits, for cones of any step length: the grids that get its workspace.
+bool tiles_possible(int nx, int ny, bool cones);
 
 // Tile geometry of the fused path.
 struct FusedGeom {

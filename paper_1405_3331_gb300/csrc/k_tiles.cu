@@ -1192,6 +1192,14 @@ bool tiles_shape(int nx, int ny, bool cones, float step_len, float h, int K, int
 
 }  // namespace
 
+bool tiles_possible(int nx, int ny, bool cones)
+{
+    TilesGeom g;
+    for (int K = 1; K <= 16; ++K)                        // (a longer step's halo is the wider: it fits no grid that none of these do)
+        if (tiles_shape(nx, ny, cones, 0.0f, 1.0f, K, kTilesMax, g)) return true;
+    return false;
+}
+
 // The steps a round K: microseconds a step by what was measured on GB300 -- a field warp's rows
 // (0.1 each; at least 0.75 with cones, their dependent chain), and an exchange shared by the K steps of a round
 // (1.9, and 0.045 a node of halo width; 1.6 times that where rows are not whole float4 groups).
