@@ -254,6 +254,28 @@ def test_crowds_on_rows_of_any_length_go_to_another_path_and_are_looked_at_again
     b.close()
 
 
+def test_a_wait_that_runs_out_is_reported_and_the_next_run_is_normal(cue):
+    """Two looks at a neighbour's packets are too few: blocks give up, the others follow, the launch ends and the
+    status says so; its tags, counts and abort word are no part of the next run."""
+    w = _case("512x384-clamp-2000cones")
+    sim = cue.Simulation(w, path=cue.CUE_PATH_PERSIST)
+    for steps in (40, 100):
+        sim.set_option(cue.CUE_OPT_WAIT_LIMIT, 1)
+        sim.sim_run(steps)
+        assert sim.status() == cue.CUE_ERR_TIMEOUT
+        assert sim.status() == cue.CUE_OK                # cleared after reporting
+    sim.set_option(cue.CUE_OPT_WAIT_LIMIT, 0)
+    sim.load(C=w.field0(), pos=w.pos, dir=w.dir, active=w.active, step=0)
+    sim.sim_run(31)
+    sim.check()
+    got = sim.snapshot()
+    sim.close()
+    ref = cue.Simulation(w, path=cue.CUE_PATH_PLAIN)
+    ref.sim_run(31)
+    _assert_same(ref.snapshot(), got)
+    ref.close()
+
+
 def test_device_side_problems_are_reported(cue):
     """Non-finite input is reported; sources outside the grid are skipped and reported."""
     w = _case("512x300")
