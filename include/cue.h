@@ -97,7 +97,9 @@ typedef struct cue_sim cue_sim;   /* opaque, host-side */
 /* ---- options (cue_set_option) ------------------------------------------ */
 #define CUE_OPT_PATH            1  /* value: CUE_PATH_*                                    */
 #define CUE_OPT_TEMPORAL_DEPTH  2  /* value: steps fused per launch on the fused path, or per
-                                      exchange of the persistent path's tile engine (1..16),
+                                      exchange of the persistent path's tile engine (1..16;
+                                      under AUTO a depth also asks for that engine wherever it
+                                      fits, unless the handle's runs crowd into few tiles),
                                       0 = library choice; on 3D handles 2 selects the
                                       blocked path under AUTO, other values the one-step
                                       kernel                                                */

@@ -1375,9 +1375,9 @@ bool tiles_supported(Sim &s)
 
 // The modelled time of a run against the other path's: short calls pay for the load of the grid and both buffers' way
 // out, large grids for tall tiles and many exchanges, crowds for a tile whose cones its block steps alone (crowd_ns), where
-// other paths share them out.  Over 288 x 256 to 1701^2, 1 to 256 steps a call, with and without cones and map, the choice
-// is the faster one or within 6% of it but for odd rows at 6 steps (18%).  The crowd's part is read back from the last
-// watched run without waiting, as the fused path's helpers are sized.
+// other paths share them out.  Of 420 measured runs (35 shapes from 129^2 to 1701^2, with and without cones and map, 1 to 256
+// steps), the choice is the faster path or within 5% of it in 410, and 20% off at worst (129^2, 6 steps: 16 us, 14 as
+// launches).  The crowd's part is read back from the last watched run without waiting, as the fused path's helpers are sized.
 bool tiles_faster(Sim &s, int nsteps, double other_us)
 {
     TilesGeom g;

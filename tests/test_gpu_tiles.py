@@ -204,6 +204,17 @@ def test_many_short_runs_find_every_cone_once(cue, name, depth, chunk):
     b.close()
 
 
+@pytest.mark.parametrize("seed", [3, 14, 15, 92])
+def test_long_runs_whose_cones_gather(cue, seed):
+    """The large endpoint configuration: its cones gather at 32 sources, in tiles that hold 128 now and 129 then, over
+    2,000 steps of 7 a round."""
+    w = W.config_c5(seed=seed, n=1024, n_src=32, n_axons=4096, nsteps=2000)
+    a, _ = _run(cue, w, cue.CUE_PATH_PLAIN, [2000])
+    b, (path, _) = _run(cue, w, cue.CUE_PATH_AUTO, [2000])
+    assert path == cue.CUE_PATH_PERSIST
+    _assert_same(a, b)
+
+
 @pytest.mark.parametrize("depth", [1, 2, 6])
 @pytest.mark.parametrize("name", ["640x400-crowd-clamp-8000cones", "640x400-crowd-stop-3000cones"])
 def test_a_crowd_that_marches_through_tiles(cue, name, depth):
